@@ -114,6 +114,41 @@ VCoef<V> make_vcoef(const lb_params& p, const lb_derived& d) {
   c.sixth = bc<V>(1.0 / 6.0);
   c.i12 = bc<V>(1.0 / 12.0);
   c.quarter = bc<V>(0.25);
+  if constexpr (std::is_same<V, double>::value) {
+    Coef64<double>& x = c.x;
+    x.G2s = d.G2 / 12.0;
+    x.lam_RT3 = 3.0 * lam * RT;
+    x.cA = 1.5 * d.G2 - 3.0 * lam * a;
+    x.cA2 = 2.0 * x.cA;
+    x.nb23 = -d.beta2 / 3.0;
+    x.hk3 = 3.0 * c.hk_seps;
+    x.nsq = -sq;
+    x.nseps = -seps;
+    x.om_e2 = 2.0 * c.om_e;
+    x.om_p2 = 2.0 * c.om_p;
+    x.nR11 = -c.R11 * c.om_e;
+    x.nR17 = -c.R17 * c.om_p;
+    x.nR18 = -c.R18 * c.om_p;
+    x.nR71 = -c.R71 * c.om_e;
+    x.nR77 = -c.R77 * c.om_p;
+    x.nR81 = -c.R81 * c.om_e;
+    x.nR88 = -c.R88 * c.om_p;
+    x.nT1a = -c.T1a / 12.0;
+    x.nT1b = c.negT1b / 12.0;
+    x.nT7 = -c.T7 / 12.0;
+    x.T7b = c.T7b / 12.0;
+    x.nT8 = c.T8 / 12.0;
+    x.Q1 = c.Q1G2 / 144.0;
+    x.Q2 = c.Q2G2 / 432.0;
+    x.Q78 = c.Q78G2 / 144.0;
+    x.third = 1.0 / 3.0;
+    x.nsixth = -1.0 / 6.0;
+    x.twelfth = 1.0 / 12.0;
+    x.ninth = 1.0 / 9.0;
+    x.i36 = 1.0 / 36.0;
+    x.ni36 = -1.0 / 36.0;
+    x.i18 = 1.0 / 18.0;
+  }
   return c;
 }
 
@@ -169,7 +204,8 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
     rnd.k = h->graph_k;
   }
   if (h->variant == LB_FUSED) {
-    const dim3 grd((nx + kTileX - 1) / kTileX, (ny + kTileY - 1) / kTileY);
+    constexpr int TY = fused_rows<V>();
+    const dim3 grd((nx + kTileX - 1) / kTileX, (ny + TY - 1) / TY);
     if constexpr (sizeof(store_t) <= 4 && std::is_same<V, f2>::value) {
       if (h->use_tma && h->use_dyn) {
         k_step_tma_dyn<V, store_t><<<h->dyn_grid, kFusedThreads, Win2<store_t>::smem, h->stream>>>(
@@ -182,7 +218,7 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
         return;
       }
     }
-    k_step_fused<V, store_t><<<grd, kFusedThreads, 0, h->stream>>>(fin, fout, nx, ny, h->st, cv, rnd);
+    k_step_fused<V, store_t><<<grd, TileShape<TY>::threads, 0, h->stream>>>(fin, fout, nx, ny, h->st, cv, rnd);
   } else {
     real* rho = static_cast<real*>(h->scratch);
     const dim3 blk(32, 8), grd((nx + 31) / 32, (ny + 7) / 8);

@@ -193,6 +193,23 @@ __device__ __forceinline__ void store9_pair(__half* p, int plane, const float (&
 }
 
 // ---------------------------------------------------------------------------
+// Constants of the FP64 collision (below) that combine several of VCoef's; empty for
+// the FP32 types.  S there is 12 times the force stencil, hence the 1/12 and 1/144.
+template <typename V>
+struct Coef64 {};
+template <>
+struct Coef64<double> {
+  double G2s;                               // G2 / 12
+  double lam_RT3, cA, cA2;                  // 3 lam R T, 3 G2 / 2 - 3 lam a, twice that
+  double nb23, hk3;                         // -beta2 / 3, 3 hk_seps
+  double nsq, nseps;                        // -s_q, -s_eps
+  double om_e2, om_p2;                      // 2 om_e, 2 om_p
+  double nR11, nR17, nR18, nR71, nR77, nR81, nR88;  // -R times om_e (columns 1) or om_p (columns 7, 8)
+  double nT1a, nT1b, nT7, T7b, nT8;         // -T1a / 12, -3 (2 - s_e)(2 k + h) / 24, -T7 / 12, (2 - s_p) b / 12, -(2 - s_p) b / 24
+  double Q1, Q2, Q78;                       // Q1G2 / 144, Q2G2 / 432, Q78G2 / 144
+  double third, nsixth, twelfth, ninth, i36, ni36, i18;
+};
+
 // Collision constants for value type V (host: make_vcoef).
 template <typename V>
 struct VCoef {
@@ -209,6 +226,7 @@ struct VCoef {
   V neg_a, eight, twenty, Q1, Q2, Q78;
   // stencil weights omega = 1/3 (axes), 1/12 (diagonals) of Eq. 12
   V third, twelfth;
+  Coef64<V> x;
 };
 
 // The coefficients that depend on the lattice's temperature, pressure scale,
@@ -377,6 +395,156 @@ __device__ __forceinline__ void collide(const VCoef<V>& c, const V (&d)[9], V Sx
   collide(c, lattice_part(c), d, Sx, Sy, o);
 }
 
+// FP64 reciprocal: one third-order step r (1 + e + e^2), e = 1 - x r (the geometric
+// series of 1 / x around r; Householder's method of order 2), on the hardware's approximation, whose residual
+// stays below 2^-19.9 (measured), so that e^3 is below 2^-59; within 1 ulp of 1 / x
+// over [2^-32, 2^32] (measured).  Three FP64 instructions.
+__device__ __forceinline__ double rcp_fp64(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = __fma_rn(-x, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
+// FP64 node: the collision above with its terms regrouped for the fewest FP64
+// instructions.  The FP64 pipe bounds every FP64 step (a warp instruction takes 19
+// cycles of an SM, add, multiply and fused multiply-add alike), so instructions are
+// what counts: about 200 per node, density and stencil included, against 222 with the
+// generic form (1024^2: 456 -> 395 us a step with the half-size tiles of k_step_fused).
+//   * one reciprocal, of rho (1 - b rho), serves 1 / rho and the EOS;
+//   * with k = J - F (J = rho u of Eq. 5), V = k.u and t_x = jx uy - Fy ux the
+//     brackets D + F_m / 2 become short: G4 = (m4 + jx) - 3 uy t_x, G1 = (m1 + 2 rho)
+//     - 2 eta - 3 V, and so on;
+//   * K1, K7, K8 of step (4) are all multiples of 3 g - 1;
+//   * the scale factors of (I - S / 2), of the stencil (S arrives as 12 S) and of
+//     M^-1 sit in the constants; o[0] follows from mass conservation.
+// rdev: the node's density deviation as phase 1 summed it.  Every operation is
+// rounded as written (no contraction), so that every kernel gets the same bits.
+struct r64 {
+  double v;
+};
+__device__ __forceinline__ r64 operator+(r64 a, r64 b) { return {__dadd_rn(a.v, b.v)}; }
+__device__ __forceinline__ r64 operator-(r64 a, r64 b) { return {__dsub_rn(a.v, b.v)}; }
+__device__ __forceinline__ r64 operator-(r64 a) { return {-a.v}; }
+__device__ __forceinline__ r64 operator*(r64 a, r64 b) { return {__dmul_rn(a.v, b.v)}; }
+__device__ __forceinline__ r64 operator*(double a, r64 b) { return {__dmul_rn(a, b.v)}; }
+__device__ __forceinline__ r64 fmav(r64 a, r64 b, r64 c) { return {__fma_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ r64 fmav(double a, r64 b, r64 c) { return {__fma_rn(a, b.v, c.v)}; }
+
+__device__ __forceinline__ void collide_fp64(const VCoef<double>& c, const double (&f)[9], double rdev_, double Sx,
+                                             double Sy, double (&o)[9]) {
+  const Coef64<double>& x = c.x;
+  const r64 d0{f[0]}, d1{f[1]}, d2_{f[2]}, d3{f[3]}, d4{f[4]}, d5{f[5]}, d6{f[6]}, d7{f[7]}, d8{f[8]};
+  const r64 rdev{rdev_}, X{Sx}, Y{Sy};
+  const r64 a13 = d1 + d3, a24 = d2_ + d4, a57 = d5 + d7, a68 = d6 + d8;
+  const r64 s13 = d1 - d3, s24 = d2_ - d4, s57 = d5 - d7, s68 = d6 - d8;
+  const r64 axis = a13 + a24, diag = a57 + a68;
+  const r64 dm = s57 - s68, dp = s57 + s68;
+  const r64 jx = s13 + dm, jy = s24 + dp;
+  const r64 P4 = fmav(2.0, dm, -s13), P6 = fmav(2.0, dp, -s24);  // m4 + jx, m6 + jy
+  const r64 m7 = a13 - a24, m8 = a57 - a68;
+  const r64 p1 = fmav(-2.0, d0, fmav(4.0, diag, axis));  // m1 + 2 rho (deviations)
+  const r64 p2 = d0 - axis;                              // (m2 - rho) / 3
+
+  // EOS: eta, 3 g - 1 (g = p_LBE' = p_EOS' + G^2 rho) and 1 / rho.
+  const r64 rho = rdev + r64{c.rho_ref};
+  r64 ir, eta, g3;
+  if (c.eos == LB_EOS_VDW) {
+    const r64 om = fmav(c.neg_bq, rho, r64{1.0});
+    const r64 r{rcp_fp64((rho * om).v)};
+    const r64 io = r * rho;
+    ir = r * om;
+    const r64 q3 = x.lam_RT3 * io;
+    eta = rho * (fmav(x.cA, rho, q3) - r64{1.0});
+    g3 = fmav(q3, io, fmav(x.cA2, rho, r64{-1.0}));
+  } else {
+    const r64 t = c.bq * rho, om = r64{1.0} - t;
+    const r64 r{rcp_fp64((rho * om).v)};
+    const r64 io = r * rho;
+    ir = r * om;
+    const r64 io3 = io * io * io, t2 = t * t;
+    const r64 z = fmav(t2, om, r64{1.0} + t) * io3;                                            // (1+t+t^2-t^3)/(1-t)^3
+    const r64 dz = fmav(t2, fmav(t, t - r64{4.0}, r64{4.0}), fmav(4.0, t, r64{1.0})) * (io3 * io);  // its rho-slope
+    eta = rho * (fmav(x.lam_RT3, z, x.cA * rho) - r64{1.0});
+    g3 = fmav(x.lam_RT3, dz, fmav(x.cA2, rho, r64{-1.0}));
+  }
+
+  // Force, velocity and their products.
+  const r64 G2r = x.G2s * rho;
+  const r64 Fx = G2r * X, Fy = G2r * Y;
+  const r64 Jx = fmav(0.5, Fx, jx), Jy = fmav(0.5, Fy, jy);
+  const r64 ux = Jx * ir, uy = Jy * ir;
+  const r64 x2 = ux * ux, y2 = uy * uy, xy = ux * uy, u2 = x2 + y2, d2 = x2 - y2;
+  const r64 bx = ux * X, by = uy * Y, e1 = uy * X, e2 = ux * Y;
+  const r64 f1 = G2r * e2, f2_ = G2r * e1, Fc = f1 + f2_;  // Fy ux, Fx uy
+  const r64 cx = G2r * bx, cy = G2r * by, Fu = cx + cy, Fd = cx - cy;
+  const r64 va = (Jx - Fx) * ux, vb = (Jy - Fy) * uy, V = va + vb, dv = va - vb;
+  const r64 z = Jx * uy;
+  const r64 ux3 = 3.0 * ux, uy3 = 3.0 * uy, xy3 = 3.0 * xy, hF = xy3 * Fc;
+
+  // (1): G = m - m_eq + F_m / 2 (g2 = G2 / 3).
+  const r64 G1 = fmav(-3.0, V, fmav(-2.0, eta, p1));
+  const r64 g2 = fmav(x.nb23, eta, fmav(-xy3, z, p2 + V)) + hF;
+  const r64 G7 = m7 - dv;
+  const r64 G8 = fmav(0.5, Fc, m8) - z;
+  const r64 G4 = fmav(-uy3, fmav(jx, uy, -f1), P4);
+  const r64 G6 = fmav(-ux3, fmav(jy, ux, -f2_), P6);
+  // Odd part: K = m + j + F + F_m - s_q G; p = the axis pair's odd half, q the diagonal's.
+  const r64 K4 = fmav(uy3, fmav(2.0, f1, f2_), fmav(x.nsq, G4, P4));
+  const r64 K6 = fmav(ux3, fmav(2.0, f2_, f1), fmav(x.nsq, G6, P6));
+  const r64 jFx = jx + Fx, jFy = jy + Fy;
+  const r64 px = fmav(x.nsixth, K4, x.third * jFx), py = fmav(x.nsixth, K6, x.third * jFy);
+  const r64 qx = x.twelfth * (jFx + K4), qy = x.twelfth * (jFy + K6);
+  // (2), (3): A / om.
+  const r64 pG = ux * G4, qG = uy * G6;
+  const r64 A1 = fmav(c.hh_sq, pG + qG, fmav(x.hk3, g2, G1));
+  const r64 A7 = fmav(c.b_sq, pG - qG, G7);
+  const r64 A8 = fmav(c.hb_sq, fmav(uy, G4, ux * G6), G8);
+  // (4) to (6).
+  const r64 uSp = e1 + e2, uSm = e1 - e2;
+  const r64 ax = x2 * bx, ay = y2 * by;
+  const r64 yg = g3 * xy;
+  const r64 q8 = g3 * fmav(u2, uSp, fmav(x2, e1, y2 * e2));
+  const r64 sxx = X * X, syy = Y * Y, ss = sxx + syy;
+  r64 X1 = fmav(3.0, fmav(2.0, Fu, V), fmav(2.0, eta, -G1));  // mbar1 + 2 rho
+  X1 = fmav(x.om_e2, A1, fmav(x.Q1, ss, X1));
+  X1 = fmav(x.nR11, u2 * A1, fmav(x.nR17, d2 * A7, fmav(x.nR18, xy * A8, X1)));
+  X1 = fmav(x.nT1a, ax + ay, fmav(x.nT1b, yg * uSp, X1));
+  r64 X2 = fmav(2.0, hF - Fu, p2);  // (mbar2 - rho) / 3
+  X2 = fmav(x.nseps, g2, fmav(x.Q2, ss, X2));
+  r64 b7 = fmav(2.0, Fd, dv - G7);  // mbar7
+  b7 = fmav(x.om_p2, A7, fmav(x.Q78, sxx - syy, b7));
+  b7 = fmav(x.nR71, d2 * A1, fmav(x.nR77, u2 * A7, b7));
+  b7 = fmav(x.nT7, ax - ay, fmav(x.T7b, yg * uSm, b7));
+  r64 b8 = fmav(2.0, z, -m8);  // mbar8
+  b8 = fmav(x.om_p2, A8, fmav(x.Q78, X * Y, b8));
+  b8 = fmav(x.nR81, xy * A1, fmav(x.nR88, u2 * A8, b8));
+  b8 = fmav(x.nT8, q8, b8);
+  // Inverse transform.
+  const r64 base_a = fmav(x.ni36, X1, fmav(x.nsixth, X2, x.ninth * rdev));
+  const r64 base_d = fmav(x.i18, X1, fmav(x.twelfth, X2, x.i36 * rdev));
+  const r64 ba7 = fmav(0.25, b7, base_a), bm7 = fmav(-0.25, b7, base_a);
+  const r64 bd8 = fmav(0.25, b8, base_d), bm8 = fmav(-0.25, b8, base_d);
+  const r64 qs = qx + qy, qd = qy - qx;
+  o[0] = fmav(-4.0, base_a + base_d, rdev).v;
+  o[1] = (ba7 + px).v;
+  o[2] = (bm7 + py).v;
+  o[3] = (ba7 - px).v;
+  o[4] = (bm7 - py).v;
+  o[5] = (bd8 + qs).v;
+  o[6] = (bm8 + qd).v;
+  o[7] = (bd8 - qs).v;
+  o[8] = (bm8 - qd).v;
+}
+
+// 12 times the force stencil, for collide_fp64 (eight instructions).
+__device__ __forceinline__ void stencil12(double ml, double mc, double mr, double cl, double cr, double pl, double pc,
+                                          double pr, double& X, double& Y) {
+  const double u = __dsub_rn(pr, ml), v = __dsub_rn(pl, mr);
+  X = __fma_rn(4.0, __dsub_rn(cr, cl), __dsub_rn(u, v));
+  Y = __fma_rn(4.0, __dsub_rn(pc, mc), __dadd_rn(u, v));
+}
+
 // Force stencil of Eq. 12 from the densities of the 8 neighbours
 // (r_<row><col>: row m/c/p = y-1/y/y+1, col l/r = x-1/x+1).
 template <typename real>
@@ -385,6 +553,23 @@ __device__ __forceinline__ void stencil(real r_ml, real r_mc, real r_mr, real r_
   const real third = real(1.0 / 3.0), twelfth = real(1.0 / 12.0);
   Sx = third * (r_cr - r_cl) + twelfth * ((r_pr - r_pl) + (r_mr - r_ml));
   Sy = third * (r_pc - r_mc) + twelfth * ((r_pr + r_pl) - (r_mr + r_ml));
+}
+
+// Stencil and collision of one node (a pair for V = f2) from the densities (deviations)
+// of the node and its neighbours: what phase 2 of every step kernel does.
+template <typename V>
+__device__ __forceinline__ void collide_node(const VCoef<V>& c, const LatCoef<V>& l, const V (&d)[9], V, V ml, V mc,
+                                             V mr, V cl, V cr, V pl, V pc, V pr, V (&o)[9]) {
+  const V Sx = fmav(c.third, cr - cl, c.twelfth * ((pr - pl) + (mr - ml)));
+  const V Sy = fmav(c.third, pc - mc, c.twelfth * ((pr + pl) - (mr + ml)));
+  collide(c, l, d, Sx, Sy, o);
+}
+__device__ __forceinline__ void collide_node(const VCoef<double>& c, const LatCoef<double>&, const double (&d)[9],
+                                             double rdev, double ml, double mc, double mr, double cl, double cr,
+                                             double pl, double pc, double pr, double (&o)[9]) {
+  double X, Y;
+  stencil12(ml, mc, mr, cl, cr, pl, pc, pr, X, Y);
+  collide_fp64(c, d, rdev, X, Y, o);
 }
 
 }  // namespace lbm

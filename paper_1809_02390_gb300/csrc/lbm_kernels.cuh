@@ -53,6 +53,11 @@ template <typename real>
 __device__ __forceinline__ real sum9(const real (&f)[9]) {
   return ((f[0] + (f[1] + f[3])) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8]));
 }
+// FP64: the rounded additions of collide_fp64, whose four pair sums are then shared.
+__device__ __forceinline__ double sum9(const double (&f)[9]) {
+  auto add = [](double a, double b) { return __dadd_rn(a, b); };
+  return add(add(add(f[0], add(f[1], f[3])), add(f[2], f[4])), add(add(f[5], f[7]), add(f[6], f[8])));
+}
 
 // Fused stream + force + collide step on a TX x TY tile (TX = 32 columns, TY
 // rows, 16 TY threads, two nodes per thread in the same column, TY/2 rows apart).
@@ -177,10 +182,15 @@ __device__ __forceinline__ void collide_nodes(const typename LaneType<V>::type (
 #pragma unroll
     for (int k = 0; k < kTileRows; ++k) {
       const int ly = M::ly(k) + 1, lx = M::lx(k) + 1;
-      real Sx, Sy;
-      stencil(rs[ly - 1][lx - 1], rs[ly - 1][lx], rs[ly - 1][lx + 1], rs[ly][lx - 1], rs[ly][lx + 1],
-              rs[ly + 1][lx - 1], rs[ly + 1][lx], rs[ly + 1][lx + 1], Sx, Sy);
-      collide(c, l, f[k], Sx, Sy, out[k]);
+      if constexpr (sizeof(real) == 8) {
+        collide_node(c, l, f[k], rs[ly][lx], rs[ly - 1][lx - 1], rs[ly - 1][lx], rs[ly - 1][lx + 1], rs[ly][lx - 1],
+                     rs[ly][lx + 1], rs[ly + 1][lx - 1], rs[ly + 1][lx], rs[ly + 1][lx + 1], out[k]);
+      } else {
+        real Sx, Sy;
+        stencil(rs[ly - 1][lx - 1], rs[ly - 1][lx], rs[ly - 1][lx + 1], rs[ly][lx - 1], rs[ly][lx + 1],
+                rs[ly + 1][lx - 1], rs[ly + 1][lx], rs[ly + 1][lx + 1], Sx, Sy);
+        collide(c, l, f[k], Sx, Sy, out[k]);
+      }
     }
   }
 }
@@ -278,15 +288,23 @@ __device__ __forceinline__ void step_tile(const store_t* __restrict__ fin, store
   collide_tile<V, store_t, TY, XP>(f, fout, nx, ny, st, c, l, x0, y0, rs, rnd);
 }
 
-template <typename V, typename store_t>
-__global__ void __launch_bounds__(kFusedThreads, fused_min_blocks<V>())
+// TY: rows of a tile.  FP64 steps take 8 (fused_rows): the FP64 pipe bounds them, so an
+// SM's time is its number of tiles, and half-size tiles spread more evenly (1024^2 on
+// 152 SMs: at most 27 of 26.9 tiles on average, against 14 of 13.5) at the price of one
+// more density addition per node.
+template <typename V>
+constexpr int fused_rows() {
+  return sizeof(typename LaneType<V>::type) == 8 ? 8 : kTileY;
+}
+template <typename V, typename store_t, int TY = fused_rows<V>()>
+__global__ void __launch_bounds__(TileShape<TY>::threads, fused_min_blocks<V>() * (kTileY / TY))
     k_step_fused(const store_t* __restrict__ fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
                  VCoef<V> c, Rounding rnd) {
   rnd = resolve(rnd);
-  __shared__ __align__(16) typename LaneType<V>::type rs[kTileY + 2][kTileX + 2];
+  __shared__ __align__(16) typename LaneType<V>::type rs[TY + 2][kTileX + 2];
   constexpr bool XP = xpairs<store_t>() && Lanes<V>::n == 2;
-  step_tile<V, store_t, kTileY, NoHook, XP>(fin, fout, nx, ny, st, c, lattice_part(c), blockIdx.x * kTileX,
-                                            blockIdx.y * kTileY, rs, NoHook(), rnd);
+  step_tile<V, store_t, TY, NoHook, XP>(fin, fout, nx, ny, st, c, lattice_part(c), blockIdx.x * kTileX,
+                                        blockIdx.y * TY, rs, NoHook(), rnd);
 }
 
 // Two-pass variant, pass 1: density plane rho_dev(x) = sum_i fbar_i(x - e_i).
@@ -314,11 +332,16 @@ __global__ void k_collide_rho(const store_t* __restrict__ fin, store_t* __restri
   const real* rm = rho + ym * nx;
   const real* rc = rho + y * nx;
   const real* rpp = rho + yp * nx;
-  real Sx, Sy;
-  stencil(__ldg(rm + xm), __ldg(rm + x), __ldg(rm + xp), __ldg(rc + xm), __ldg(rc + xp), __ldg(rpp + xm),
-          __ldg(rpp + x), __ldg(rpp + xp), Sx, Sy);
+  const real ml = __ldg(rm + xm), mc = __ldg(rm + x), mr = __ldg(rm + xp), cl = __ldg(rc + xm), cr = __ldg(rc + xp);
+  const real pl = __ldg(rpp + xm), pc = __ldg(rpp + x), pr = __ldg(rpp + xp);
   real o[9];
-  collide(c, f, Sx, Sy, o);
+  if constexpr (sizeof(real) == 8) {
+    collide_node(c, lattice_part(c), f, __ldg(rc + x), ml, mc, mr, cl, cr, pl, pc, pr, o);
+  } else {
+    real Sx, Sy;
+    stencil(ml, mc, mr, cl, cr, pl, pc, pr, Sx, Sy);
+    collide(c, f, Sx, Sy, o);
+  }
   store9(fout + st.at(0, x, y), st.ps, o, x, y, nx, rnd);
 }
 
