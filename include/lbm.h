@@ -132,7 +132,10 @@ int lb_derive(const lb_params* p, lb_derived* out);
 size_t lb_state_bytes(const lb_params* p);
 
 /* Bytes of device scratch memory: one density plane (two-pass variant, reductions),
- * the reduction workspace and 256 bytes of tile tickets (fused tensor-copy step). */
+ * the reduction workspace, 256 bytes of tile tickets (fused tensor-copy step) and, for
+ * lattices that fit the SMs' shared memory, the exchange words of the resident run
+ * (lb_step; at most 8 MB).  A buffer without the last part is accepted too: lb_step
+ * then launches step by step. */
 size_t lb_scratch_bytes(const lb_params* p);
 
 /* Creates a handle bound to the caller's buffers and stream and initialises the
@@ -155,7 +158,11 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
             size_t scratch_bytes, const double* rho0, int rho0_on_device, void* stream);
 
 /* Advances nsteps >= 0 time steps (Eq. 13 + supplement Eq. 2) on the stream.
- * Asynchronous.  Runs of 64 steps replay a CUDA graph that the handle captures on
+ * Asynchronous.  A fused lattice whose populations fit the SMs' shared memory twice
+ * (FP64 to about 485^2, FP32 610^2, FP16 860^2) takes calls of at least four steps in
+ * one cooperative launch that keeps it there (same bits; waits between its blocks are
+ * bounded at 10 s and reported by lb_status), unless lb_set_step_blocks or
+ * lb_set_tile_dispatch ask for another form.  Else runs of 64 steps replay a CUDA graph that the handle captures on
  * first use (again after lb_set_step_blocks or lb_set_tile_dispatch change the
  * launch); the graph runs on a stream the handle owns, ordered after the caller's
  * stream's earlier work and before its later work, and gives the same bits as 64

@@ -191,6 +191,10 @@ size_t rho_plane_bytes(const lb_params* p) {
 size_t reduce_bytes() { return size_t(kMaxReduceBlocks) * kReduceSlots * sizeof(double) + 256; }
 constexpr size_t kQueueBytes = 256;  // tile tickets of the dynamic tensor-copy step
 
+// Scratch without the exchange buffer of the resident run: enough for every call (the
+// steps are then launched one by one).
+size_t base_scratch_bytes(const lb_params* p) { return rho_plane_bytes(p) + reduce_bytes() + kQueueBytes; }
+
 template <typename V, typename real, typename store_t>
 void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
   const store_t* fin = static_cast<const store_t*>(h->f[h->cur]);
@@ -479,6 +483,13 @@ int configure(lb_handle* h) {
     LB_CUDA(h, cudaMemsetAsync(h->queue, 0, 2 * sizeof(unsigned), h->stream));
     h->use_dyn = true;
   }
+  // Resident run: needs its exchange buffer behind the rest of the scratch.
+  void* mail = nullptr;
+  const size_t base = base_scratch_bytes(&h->p);
+  if (h->scratch && h->scratch_bytes >= base + res_mail_bytes(h->p.nx, h->p.ny) &&
+      reinterpret_cast<uintptr_t>(h->scratch) % 16 == 0)
+    mail = static_cast<char*>(h->scratch) + base;
+  LB_CUDA(h, res_configure(h, mail));
   return LB_OK;
 }
 
@@ -550,7 +561,7 @@ size_t lb_state_bytes(const lb_params* p) {
 
 size_t lb_scratch_bytes(const lb_params* p) {
   if (!p || p->nx < 1 || p->ny < 1) return 0;
-  return rho_plane_bytes(p) + reduce_bytes() + kQueueBytes;
+  return base_scratch_bytes(p) + res_mail_bytes(p->nx, p->ny);
 }
 
 int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scratch, size_t scratch_bytes,
@@ -564,9 +575,9 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
   if (!f_a || !f_b || f_a == f_b) return fail(nullptr, LB_EINVAL, "f_a and f_b must be two distinct device buffers");
   if (!rho0) return fail(nullptr, LB_EINVAL, "null initial density");
   const int variant = p->variant == LB_TWO_PASS ? LB_TWO_PASS : LB_FUSED;
-  if (scratch && scratch_bytes < lb_scratch_bytes(p))
+  if (scratch && scratch_bytes < base_scratch_bytes(p))
     return fail(nullptr, LB_ENOMEM, "scratch of %zu bytes is below the %zu needed", scratch_bytes,
-                lb_scratch_bytes(p));
+                base_scratch_bytes(p));
   if (variant == LB_TWO_PASS && !scratch)
     return fail(nullptr, LB_ENOMEM, "the two-pass variant needs %zu bytes of scratch", lb_scratch_bytes(p));
   const size_t N = size_t(p->nx) * p->ny;
@@ -669,6 +680,8 @@ namespace {
 
 // Steps per captured graph (even, so a replay ends on the buffer it started from).
 constexpr int kStepGraph = 64;
+// Fewest steps of a call that run resident.
+constexpr int64_t kResMinSteps = 4;
 
 void launch_one_step(lb_handle* h) {
   switch (h->p.precision) {
@@ -743,6 +756,10 @@ int lb_step(lb_handle* h, int64_t nsteps) {
   if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
+  }
+  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= kResMinSteps && capture == cudaStreamCaptureStatusNone) {
+    LB_CUDA(h, res_run(h, nsteps, nullptr));
+    return LB_OK;
   }
   if (nsteps >= kStepGraph && !h->graph_off && capture == cudaStreamCaptureStatusNone) {
     if (!ensure_step_graph(h)) {
@@ -911,6 +928,7 @@ int lb_set_step_blocks(lb_handle* h, int blocks) {
   const int tiles = ((h->p.nx + kTileX - 1) / kTileX) * ((h->p.ny + kTileY - 1) / kTileY);
   h->tma_grid = blocks == 0 ? h->tma_grid_auto : (blocks < tiles ? blocks : tiles);
   h->dyn_grid = blocks == 0 ? h->dyn_grid_auto : (blocks < tiles ? blocks : tiles);
+  h->forced_blocks = blocks != 0;
   return LB_OK;
 }
 
@@ -919,6 +937,7 @@ int lb_set_tile_dispatch(lb_handle* h, int dynamic) {
   if (dynamic && !(h->use_tma && h->queue))
     return fail(h, LB_ENOTSUP, "dynamic dispatch needs the tensor-copy step and the scratch buffer");
   h->use_dyn = dynamic != 0;
+  h->forced_walk = h->use_tma && !dynamic;
   return LB_OK;
 }
 

@@ -6,6 +6,19 @@
 
 #include "lbm_kernels.cuh"
 
+namespace lbm {
+// Cut of an nx x ny lattice into gx x gy tiles (tile b: columns [b nx / gx, (b + 1) nx / gx)),
+// all at least four nodes wide and high unless the lattice itself is smaller.
+struct ResPlan {
+  int gx, gy;
+  int wmax, hmax;    // largest tile
+  int pitch;         // row pitch of a tile and its halo in shared memory
+  int threads;       // of a block
+  unsigned smem;     // dynamic shared memory of a block
+  size_t words;      // 16-byte words of one parity of the exchange buffer, all tiles
+};
+}  // namespace lbm
+
 struct lb_handle {
   lb_params p;
   lb_derived d;
@@ -35,6 +48,13 @@ struct lb_handle {
   cudaGraphExec_t graph[2];
   long long graph_cfg[2];
   bool graph_off;         // capture failed once: direct launches only
+  // Resident run (lbm_resident.cu): many steps per launch on lattices that fit the SMs'
+  // shared memory.
+  bool use_res;
+  bool forced_blocks, forced_walk;  // lb_set_step_blocks, lb_set_tile_dispatch fixed another launch form
+  lbm::ResPlan res;
+  void* res_mail;         // exchange words (end of the scratch buffer)
+  unsigned res_epoch;     // numbers up to this one have been used
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
   int graph_k;            // while capturing: the place of the launch in the graph (else -1)
   lbm::VCoef<float> cf;  // FP32 scalar (two-pass variant, moments)
@@ -53,6 +73,16 @@ bool encode_population_map(CUtensorMap* map, void* base, int nx, int ny, int sx,
 // 3-D map (x, y, plane) of `planes` FP32 planes of nx x ny, box cols x rows x 1
 // (lbm_capi.cu); false if the buffer does not allow one.
 bool encode_plane_map(CUtensorMap* map, const void* base, int nx, int ny, int planes, int cols, int rows);
+// Cut of a lattice for the resident run; false if it does not fit (lbm_resident.cu).
+bool res_plan(int nx, int ny, int precision, ResPlan* out);
+// Bytes of the exchange buffer (0 when no precision of this size runs resident).
+size_t res_mail_bytes(int nx, int ny);
+// Decides whether the handle can run resident and clears the exchange buffer `mail`
+// (device memory of res_mail_bytes, 16-byte aligned, or null).
+cudaError_t res_configure(lb_handle* h, void* mail);
+// Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
+// null): device memory that receives the state after each step, one after the other.
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec);
 // Device address of lb_reduce_static's static scratch on the current device
 // (looked up once per device, which commits the array there; lbm_static.cu).
 int static_scratch_address(lb_handle* h, void** out);

@@ -1,0 +1,170 @@
+// Host side of the resident run (lbm_resident.cuh): the cut of a lattice into tiles,
+// the exchange buffer's size and the cooperative launch.
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include "lbm_resident.cuh"
+#include "lbm_handle.cuh"
+
+namespace lbm {
+
+namespace {
+
+template <typename V, typename S>
+constexpr const void* kernel_of() {
+  return reinterpret_cast<const void*>(k_resident<V, S>);
+}
+
+const void* res_kernel(int precision) {
+  switch (precision) {
+    case LB_FP64: return kernel_of<double, double>();
+    case LB_FP32: return kernel_of<f2, float>();
+    default: return kernel_of<f2, __half>();
+  }
+}
+
+size_t res_smem(int precision, int wmax, int hmax, int pitch) {
+  const size_t plane = size_t(pitch) * (hmax + 4);
+  const size_t real = precision == LB_FP64 ? 8 : 4, store = precision == LB_FP64 ? 8 : precision == LB_FP32 ? 4 : 2;
+  return size_t(res_table_bytes(wmax, hmax, precision == LB_FP64 ? 1 : 2)) + plane * (real + 18 * store);
+}
+
+}  // namespace
+
+// The cut with the smallest estimated step: a block's warps take the collision in
+// turn (FP64: 19 cycles of an SM per warp instruction, four warps at a time; FP32:
+// about 130 cycles of an SM per warp of pairs, and no less than the latency of one),
+// and each edge node costs its share of the exchange.
+bool res_plan(int nx, int ny, int precision, ResPlan* out) {
+  const bool fp64 = precision == LB_FP64;
+  const int lanes = fp64 ? 1 : 2;
+  const int max_threads = fp64 ? ResTraits<double>::max_threads : ResTraits<float>::max_threads;
+  double best = 0.0;
+  bool found = false;
+  for (int gx = 1; gx <= kResTiles && (gx == 1 || nx / gx >= 4); ++gx) {
+      int gy = kResTiles / gx;
+      if (gy > ny / 4) gy = ny / 4;
+      if (gy < 1) gy = 1;
+      const int w = (nx + gx - 1) / gx, h = (ny + gy - 1) / gy;
+      if (nx / gx < 2 || ny / gy < 2) continue;
+      if ((long long)(w + 4) * (h + 4) > 65535) continue;
+      // Warps run along the inner rows of w - 4 nodes: with a pitch that is w - 4 modulo
+      // the 32 banks, a warp that crosses into the next row stays free of conflicts
+      // (512^2 FP32: 4.54 -> 4.34 us a step), where the shared memory allows it.
+      int pitch = w > 4 ? w - 4 + (w + 4 - (w - 4) + 31) / 32 * 32 : w + 4;
+      if (res_smem(precision, w, h, pitch) > kResSmem - 1024) pitch = w + 4;
+      if (res_smem(precision, w, h, pitch) > kResSmem - 1024) continue;
+      const int items = res_slots(w, h, lanes).total;
+      const int warps = (items + 31) / 32;
+      const double work = fp64 ? 15000.0 * ((warps + 3) / 4) : (130.0 * warps > 900.0 ? 130.0 * warps : 900.0);
+      const double cost = work + 4.0 * (w + h) + 0.01 * gx * gy;
+      if (found && cost >= best) continue;
+      best = cost;
+      found = true;
+      const int rounds = (items + max_threads - 1) / max_threads;
+      int threads = ((items + rounds - 1) / rounds + 31) / 32 * 32;
+      if (threads < 128) threads = 128;
+      *out = ResPlan{gx, gy, w, h, pitch, threads, unsigned(res_smem(precision, w, h, pitch)),
+                     size_t(gx) * gy * 6 * (w + h) * (fp64 ? 2 : 1)};
+    }
+  return found;
+}
+
+// Largest over the precisions, so that the scratch size differs between them by the
+// density plane alone.
+size_t res_mail_bytes(int nx, int ny) {
+  size_t words = 0;
+  for (int precision : {int(LB_FP64), int(LB_FP32), int(LB_FP16S)}) {
+    ResPlan p;
+    if (res_plan(nx, ny, precision, &p) && p.words > words) words = p.words;
+  }
+  return 2 * words * sizeof(uint4);
+}
+
+cudaError_t res_configure(lb_handle* h, void* mail) {
+  h->use_res = false;
+  ResPlan p;
+  if (!mail || h->variant != LB_FUSED || !res_plan(h->p.nx, h->p.ny, h->p.precision, &p)) return cudaSuccess;
+  const void* k = res_kernel(h->p.precision);
+  int dev = 0, coop = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  // The limit is the kernel's, not the handle's: always the largest any plan needs.
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kResSmem - 1024));
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, p.threads, p.smem);
+  if (e != cudaSuccess) return e;
+  if (!coop || per_sm < 1 || sms < p.gx * p.gy) return cudaSuccess;
+  e = cudaMemsetAsync(mail, 0, 2 * p.words * sizeof(uint4), h->stream);
+  if (e != cudaSuccess) return e;
+  h->res = p;
+  h->res_mail = mail;
+  h->res_epoch = 0;
+  h->use_res = true;
+  return cudaSuccess;
+}
+
+namespace {
+
+template <typename V, typename S>
+cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout, void* rec, long long rec_stride,
+                   int nsteps) {
+  const ResPlan& p = h->res;
+  ResArgs<S> a{static_cast<const S*>(fin),
+               static_cast<S*>(fout),
+               static_cast<S*>(rec),
+               rec_stride,
+               static_cast<uint4*>(h->res_mail),
+               h->wait_error,
+               h->res_epoch,
+               unsigned(h->steps),
+               nsteps,
+               h->p.nx,
+               h->p.ny,
+               p.gx,
+               p.gy,
+               p.wmax,
+               p.hmax,
+               p.pitch,
+               h->p.rounding == LB_ROUND_STOCHASTIC,
+               h->st};
+  VCoef<V> cc = c;
+  void* args[] = {&a, &cc};
+  return cudaLaunchCooperativeKernel(kernel_of<V, S>(), dim3(p.gx * p.gy), dim3(p.threads), args, p.smem, h->stream);
+}
+
+}  // namespace
+
+// Steps of one launch: a few milliseconds, so that other work on the GPU gets its turn.
+constexpr int64_t kResChunk = 4096;
+
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec) {
+  const long long stride = 9ll * h->p.nx * h->p.ny;
+  const size_t elem = h->p.precision == LB_FP64 ? 8 : h->p.precision == LB_FP32 ? 4 : 2;
+  while (nsteps > 0) {
+    // Never a launch of one step: it could not write its result in place.
+    int64_t n = nsteps <= kResChunk ? nsteps : (nsteps == kResChunk + 1 ? kResChunk - 2 : kResChunk);
+    if (h->res_epoch > 0xf0000000u) {
+      const cudaError_t e = cudaMemsetAsync(h->res_mail, 0, 2 * h->res.words * sizeof(uint4), h->stream);
+      if (e != cudaSuccess) return e;
+      h->res_epoch = 0;
+    }
+    const void* in = h->f[h->cur];
+    void* out = h->f[n & 1 ? 1 - h->cur : h->cur];
+    cudaError_t e;
+    switch (h->p.precision) {
+      case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, stride, int(n)); break;
+      case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, stride, int(n)); break;
+      default: e = launch<f2, __half>(h, h->c2, in, out, rec, stride, int(n)); break;
+    }
+    if (e != cudaSuccess) return e;
+    if (rec) rec = static_cast<char*>(rec) + size_t(n) * stride * elem;
+    h->res_epoch += unsigned(n);
+    h->steps += n;
+    if (n & 1) h->cur = 1 - h->cur;
+    nsteps -= n;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace lbm
