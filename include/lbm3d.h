@@ -98,6 +98,10 @@ int lb_d3_moments(lb_d3_handle* h, void* rho, void* ux, void* uy, void* uz);
  * that lb_d3_init allocates. */
 int lb_d3_reduce(lb_d3_handle* h, double out[8]);
 
+/* Synchronous health check: LB_ETIMEOUT if a bounded wait of the step's tensor copies
+ * gave up since the last call (the flag is cleared), else LB_OK. */
+int lb_d3_status(lb_d3_handle* h);
+
 /* Device buffer holding the current state (f_a or f_b). */
 void* lb_d3_state(const lb_d3_handle* h);
 

@@ -110,6 +110,7 @@ SIGNATURES = [
     ("lb_d3_step", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_d3_moments", ctypes.c_int, [_V, _V, _V, _V, _V]),
     ("lb_d3_reduce", ctypes.c_int, [_V, _D]),
+    ("lb_d3_status", ctypes.c_int, [_V]),
     ("lb_d3_state", _V, [_V]),
     ("lb_d3_get_state", ctypes.c_int, [_V, _V]),
     ("lb_d3_set_state", ctypes.c_int, [_V, _V]),

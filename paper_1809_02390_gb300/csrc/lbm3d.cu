@@ -15,6 +15,7 @@
 
 #include "lbm3d.h"
 #include "lbm_internal.h"
+#include "lbm_handle.cuh"
 
 #include "lbm3d_step.cuh"
 
@@ -151,9 +152,15 @@ struct lb_d3_handle {
   void* f[2];
   int cur;
   cudaStream_t stream;
-  C3<double> c64;
-  C3<float> c32;
-  int tz;  // planes per z-chunk of the step kernel
+  CV3<r64> c64;
+  CV3<f2> c32;
+  C3<float> cpull;  // of k_d3_pull
+  bool vec;         // rows of a multiple of 16 bytes (and both buffers aligned)
+  bool windows;     // k_d3_step (else k_d3_pull)
+  bool have_maps;   // tensor maps of both buffers
+  CUtensorMap maps[2];
+  int* wait_error;  // device word set by a bounded wait that gave up (behind `part`)
+  int tw, th, tz;  // tile of the step kernel and planes of its z-chunks
   // Graphs of kD3GraphSteps steps starting from buffer 0 and 1 (captured on first
   // use on the handle's private stream, launched on `stream`); graph_failed: a
   // capture failed once, so plain launches are used from then on.
@@ -247,40 +254,182 @@ C3<T> make_c3(const lb_params& p, const lb_derived& d) {
   return c;
 }
 
-// Planes per z-chunk: 32 (fewest halo planes) unless that leaves fewer than two
-// waves of resident blocks (3 per SM); then halved down to 2, because a block walks
-// its chunk plane after plane and a short grid leaves the GPU waiting on that chain.
-int chunk_planes(int nx, int ny, int nz, int sms) {
-  const long long xy = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
-  int tz = TZ;
+template <typename V>
+CV3<V> make_cv3(const lb_params& p, const lb_derived& d) {
+  auto m = [](double v) { return Val<V>::make(v); };
+  const double om_e = d.s_e / 2.0 - 1.0, om_p = d.s_p / 2.0 - 1.0;
+  const double bq = d.b * d.s_q * om_p, s_m = d.s_q, s_pi = d.s_eps;
+  const double RT = p.R_gas * d.T, cA = 1.5 * d.G2 - 3.0 * d.lam * p.eos_a;
+  CV3<V> c;
+  c.eos = p.eos;
+  c.rho_ref = m(p.rho_ref);
+  c.nbq = m(p.eos == LB_EOS_VDW ? -p.eos_b : -p.eos_b / 4.0);
+  c.lam_RT3 = m(3.0 * d.lam * RT);
+  c.cA = m(cA);
+  c.G2s = m(d.G2 / 12.0);
+  c.gq = m(d.G2 / 1728.0);
+  c.se = m(d.s_e);
+  c.kse = m(d.k * d.s_eps * om_e / 19.0);
+  c.hq = m(d.h * d.s_q * om_e * 5.0 / 57.0);
+  c.ceta = m(-(d.beta2 + 5.5));
+  c.seps_a = m(d.s_eps / 10.5);
+  c.sp3 = m(d.s_p / 3.0);
+  c.spi3 = m(s_pi / 3.0);
+  c.bq2 = m(bq * 10.0 / 3.0);
+  c.bq23 = m(bq * 10.0 / 9.0);
+  c.nbq23 = m(-bq * 10.0 / 9.0);
+  c.nsp = m(-d.s_p);
+  c.nbq5 = m(-bq * 5.0 / 3.0);
+  c.sq6 = m(d.s_q / 6.0);
+  c.om8 = m((1.0 - s_m) / 8.0);
+  c.one = m(1.0);
+  c.two = m(2.0);
+  c.three = m(3.0);
+  c.half = m(0.5);
+  c.quarter = m(0.25);
+  c.nquarter = m(-0.25);
+  c.eighth = m(0.125);
+  c.n2 = m(-2.0);
+  c.n3 = m(-3.0);
+  c.n4 = m(-4.0);
+  c.nhalf = m(-0.5);
+  c.nthird = m(-1.0 / 3.0);
+  c.sixth = m(1.0 / 6.0);
+  c.n12 = m(-1.0 / 12.0);
+  c.i24 = m(1.0 / 24.0);
+  c.n2h = m(-2.5);
+  c.n5h = m(-5.5);
+  c.n10h = m(-10.5);
+  c.c1375 = m(13.75);
+  c.c1121 = m(11.0 / 21.0);
+  return c;
+}
+
+// Planes per z-chunk (at most `most`) of a lattice of xy tiles, and the time of a step in
+// planes of a block.  A block costs its planes and `extra` more (the two planes whose
+// densities alone it needs).  The blocks start in order as places fall free: whole
+// rounds of the full chunks, then the chunks of the remainder, which go first into the
+// places that the last round leaves.  64^3 FP32 (us a step): 4 planes 14.1, 3 planes
+// 17.9; 96^3: 12 planes 33.4, 6 planes 37.3; 128^3: 14 planes 74.9, 16 planes 79.8.
+double chunk_planes(long long xy, int nz, int places, int most, double extra, int* tz_out) {
+  double best_cost = 1e300;
+  for (int tz = 1; tz <= nz && tz <= most; ++tz) {
+    const long long full = xy * (nz / tz), rounds = full / places, over = full % places;
+    const int rem = nz % tz;
+    const double d1 = tz + extra, d2 = rem + extra;
+    double cost = double(rounds + (over ? 1 : 0)) * d1;
+    if (rem) {
+      const long long room = over ? (places - over) * (long long)(d1 / d2) : 0;
+      if (xy > room) cost += double((xy - room + places - 1) / places) * d2;
+    }
+    if (cost < best_cost) {
+      best_cost = cost;
+      *tz_out = tz;
+    }
+  }
+  return best_cost;
+}
+
+// Tile and chunk of the step.  FP32: 32 x 8 tiles.  FP64: the FP64 pipe bounds the step, a
+// plane of a block takes as long as its schedulers' largest number of warps, and the SM
+// with the most planes ends last; so the tile of at most 256 nodes (even width, for the
+// 16-byte copies) and the chunk with the least time are taken: 120 x 100 x 71 in chunks of
+// 10 x 25 x 23 nodes, 539 us a step, against 607 with 32 x 8 x 5; 33 x 77 x 50 in chunks
+// of 12 x 10 x 8, 104 us against 168.
+template <typename T>
+void tile_plan(lb_d3_handle* h, int sms) {
+  using W = Win3<T>;
+  const int nx = h->p.nx, ny = h->p.ny, nz = h->nz;
+  auto tiles = [&](int tw, int th) { return (long long)((nx + tw - 1) / tw) * ((ny + th - 1) / th); };
+  h->tw = TX;
+  h->th = TY;
+  if (W::fixed) {
+    chunk_planes(tiles(TX, TY), nz, sms * d3_blocks<T>(), 32, 1.2, &h->tz);
+    return;
+  }
+  double best = 1e300;
+  for (int tw = 8; tw <= 64; tw += 2)
+    for (int th = 4; th * tw <= W::threads && th <= 32; ++th) {
+      if ((th + 2) * (tw + 2 * W::run) > W::cells || (th + 2) * (tw + 2 * W::run) / W::run > W::threads) continue;
+      if ((th + 2) * (tw + 2) > W::ring_cells || 2 * (tw + 2) + 2 * th > W::threads) continue;
+      // Warps a scheduler works off per plane: nodes, and 18 of about 300 instructions for the ring.
+      const double plane = (tw * th + 127) / 128 + 0.06 * ((2 * (tw + 2) + 2 * th + 127) / 128);
+      if (plane * double(tiles(tw, th)) * nz / (sms * d3_blocks<T>()) >= best) continue;  // even if spread evenly
+      int tz = 1;
+      const double cost = plane * chunk_planes(tiles(tw, th), nz, sms * d3_blocks<T>(), nz, 0.4, &tz);
+      if (cost < best * 0.999) {
+        best = cost;
+        h->tw = tw;
+        h->th = th;
+        h->tz = tz;
+      }
+    }
+}
+
+// k_d3_pull: 32 planes (fewest halo planes) unless that leaves fewer than two waves of
+// resident blocks (3 per SM); then halved down to 2.
+int chunk_planes_pull(int nx, int ny, int nz, int sms) {
+  const long long xy = (long long)((nx + TX - 1) / TX) * ((ny + kPullTY - 1) / kPullTY);
+  int tz = kPullTZ;
   while (tz > 2 && xy * ((nz + tz - 1) / tz) < 2LL * 3 * sms) tz /= 2;
   return tz;
 }
 
+// The step's windows by tensor copies where possible (FP32), else by 16-byte copies.
+template <typename T>
+cudaError_t configure_step(lb_d3_handle* h) {
+  h->vec = (size_t(h->p.nx) * sizeof(T)) % 16 == 0 && reinterpret_cast<uintptr_t>(h->f[0]) % 16 == 0 &&
+           reinterpret_cast<uintptr_t>(h->f[1]) % 16 == 0;
+  // FP32 lattices that k_d3_pull steps faster: rows that are no multiple of 16 bytes or
+  // shorter than a window (24 x 31 x 200: 11.5 us a step against 13.3), or so few of them
+  // that the last 32 x 8 tile is largely empty (160 x 12 x 80: 10.8 against 11.7; the
+  // windows gain 5 to 20% on full tiles).
+  const int rows8 = (h->p.ny + TY - 1) / TY * TY, rows4 = (h->p.ny + kPullTY - 1) / kPullTY * kPullTY;
+  h->windows = sizeof(T) == 8 || (h->vec && h->p.nx >= Win3<T>::cols && 10 * rows8 <= 11 * rows4);
+  h->have_maps = false;
+  std::memset(h->maps, 0, sizeof(h->maps));
+  using W = Win3<T>;
+  if (W::tensor && h->windows && h->p.ny >= W::rows) {
+    h->have_maps = true;
+    for (int k = 0; k < 2; ++k)
+      h->have_maps = h->have_maps &&
+                     encode_volume_map(&h->maps[k], h->f[k], h->p.nx, h->p.ny, h->nz, Q, W::cols, W::rows);
+  }
+  cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_d3_step<T, true>),
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, int(Win3<T>::smem));
+  if (e == cudaSuccess && sizeof(T) == 8)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_d3_step<T, sizeof(T) != 8>),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(Win3<T>::smem));
+  return e;
+}
+
+template <typename T, bool VEC>
+void launch_windows(lb_d3_handle* h, const CV3<typename ValOf<T>::V>& c) {
+  const lb_params& p = h->p;
+  const dim3 grid((p.nx + h->tw - 1) / h->tw, (p.ny + h->th - 1) / h->th, (h->nz + h->tz - 1) / h->tz);
+  k_d3_step<T, VEC><<<grid, Win3<T>::threads, Win3<T>::smem, h->stream>>>(
+      static_cast<const T*>(h->f[h->cur]), static_cast<T*>(h->f[1 - h->cur]), p.nx, p.ny, h->nz, h->tw,
+      h->th, h->tz, c, h->maps[h->cur], h->have_maps ? 1 : 0, h->wait_error);
+}
+
 void launch_step(lb_d3_handle* h) {
   const lb_params& p = h->p;
-  const int tz = h->tz;
-  const dim3 grid((p.nx + TX - 1) / TX, (p.ny + TY - 1) / TY, (h->nz + tz - 1) / tz), block(TX, TY);
-  const void* in = h->f[h->cur];
-  void* out = h->f[1 - h->cur];
-  // 32-bit plane offsets while 19 nx ny nz < 2^31 (the common case), 64-bit above.
-  const bool wide = int64_t(Q) * p.nx * p.ny * h->nz >= (int64_t(1) << 31);
-  const double* i64 = static_cast<const double*>(in);
-  const float* i32 = static_cast<const float*>(in);
   if (p.precision == LB_FP64) {
-    if (wide)
-      k_d3_step<double, false, long long><<<grid, block, 0, h->stream>>>(i64, static_cast<double*>(out), p.nx, p.ny,
-                                                                         h->nz, tz, h->c64);
+    if (h->vec)
+      launch_windows<double, true>(h, h->c64);
     else
-      k_d3_step<double, false, int><<<grid, block, 0, h->stream>>>(i64, static_cast<double*>(out), p.nx, p.ny, h->nz,
-                                                                   tz, h->c64);
+      launch_windows<double, false>(h, h->c64);
+  } else if (h->windows) {
+    launch_windows<float, true>(h, h->c32);
   } else {
-    if (wide)
-      k_d3_step<float, true, long long><<<grid, block, 0, h->stream>>>(i32, static_cast<float*>(out), p.nx, p.ny,
-                                                                       h->nz, tz, h->c32);
+    const dim3 grid((p.nx + TX - 1) / TX, (p.ny + kPullTY - 1) / kPullTY, (h->nz + h->tz - 1) / h->tz);
+    const float* in = static_cast<const float*>(h->f[h->cur]);
+    float* out = static_cast<float*>(h->f[1 - h->cur]);
+    // 32-bit plane offsets while 19 nx ny nz < 2^31, 64-bit above.
+    if (int64_t(Q) * p.nx * p.ny * h->nz >= (int64_t(1) << 31))
+      k_d3_pull<long long><<<grid, dim3(TX, kPullTY), 0, h->stream>>>(in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
     else
-      k_d3_step<float, true, int><<<grid, block, 0, h->stream>>>(i32, static_cast<float*>(out), p.nx, p.ny, h->nz, tz,
-                                                                 h->c32);
+      k_d3_pull<int><<<grid, dim3(TX, kPullTY), 0, h->stream>>>(in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
   }
   h->cur = 1 - h->cur;
 }
@@ -406,20 +555,39 @@ int lb_d3_init(lb_d3_handle** out, const lb_params* p, int32_t nz, void* f_a, vo
   h->f[1] = f_b;
   h->cur = 0;
   h->stream = s;
-  h->c64 = c;
-  h->c32 = make_c3<float>(q, d);
+  h->c64 = make_cv3<r64>(q, d);
+  h->c32 = make_cv3<f2>(q, d);
+  h->cpull = make_c3<float>(q, d);
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     sms = 152;
   }
-  h->tz = chunk_planes(q.nx, q.ny, nz, sms);
   h->err[0] = 0;
-  if (cudaMalloc(&h->part, (kReduceBlocks3 + 1) * kReduceSlots3 * sizeof(double)) != cudaSuccess) {
+  auto give_up = [&](cudaError_t ce, const char* what) {
+    cudaGetLastError();
+    delete h;
+    return cuda_fail(ce, what);
+  };
+  e = q.precision == LB_FP64 ? configure_step<double>(h) : configure_step<float>(h);
+  if (e != cudaSuccess) return give_up(e, "step configuration");
+  if (!h->windows)
+    h->tz = chunk_planes_pull(q.nx, q.ny, nz, sms);
+  else if (q.precision == LB_FP64)
+    tile_plan<double>(h, sms);
+  else
+    tile_plan<float>(h, sms);
+  if (cudaMalloc(&h->part, (kReduceBlocks3 + 2) * kReduceSlots3 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     delete h;
     return fail3(nullptr, LB_ENOMEM, "cudaMalloc of the %zu-byte reduction workspace",
-                 size_t(kReduceBlocks3 + 1) * kReduceSlots3 * sizeof(double));
+                 size_t(kReduceBlocks3 + 2) * kReduceSlots3 * sizeof(double));
+  }
+  h->wait_error = reinterpret_cast<int*>(h->part + (kReduceBlocks3 + 1) * kReduceSlots3);
+  e = cudaMemsetAsync(h->wait_error, 0, sizeof(int), s);
+  if (e != cudaSuccess) {
+    cudaFree(h->part);
+    return give_up(e, "cudaMemsetAsync of the wait word");
   }
   *out = h;
   return LB_OK;
@@ -491,6 +659,16 @@ int lb_d3_reduce(lb_d3_handle* h, double out[8]) {
   if (e != cudaSuccess) return fail3(h, LB_ECUDA, "reduction: %s", cudaGetErrorString(e));
   if (out[7] > 0) return fail3(h, LB_ENONFINITE, "%.0f nodes have a non-finite density", out[7]);
   return LB_OK;
+}
+
+int lb_d3_status(lb_d3_handle* h) {
+  if (!h) return fail3(nullptr, LB_EINVAL, "null handle");
+  int v = 0;
+  cudaError_t e = cudaMemcpyAsync(&v, h->wait_error, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess && v) e = cudaMemsetAsync(h->wait_error, 0, sizeof(int), h->stream);
+  if (e != cudaSuccess) return fail3(h, LB_ECUDA, "status: %s", cudaGetErrorString(e));
+  return v ? fail3(h, LB_ETIMEOUT, "a bounded wait for a tensor copy gave up") : LB_OK;
 }
 
 void* lb_d3_state(const lb_d3_handle* h) { return h ? h->f[h->cur] : nullptr; }

@@ -3,22 +3,21 @@
 // constants, collision constants, the node collision and the z-marching step
 // kernel.  Included by lbm3d.cu (one translation unit).
 //
-// One launch per time step: each block owns a 32 x 4 column of the x-y plane and
-// marches through a chunk of up to 32 z-planes.  For every plane it pulls the
-// populations of its nodes (pull streaming, supplement Eq. 2), sums them into the
-// density and puts the density, with a one-node ring in x and y, into a
-// three-plane ring buffer in shared memory; the collision of plane z runs once
-// plane z + 1 is there, so the force stencil (Eq. 12) of every node reads its 18
-// neighbours' densities from shared memory.  In FP32 the populations stay in
-// registers and the pulls of plane z + 2 are in flight while plane z collides; in
-// FP64 the populations of the plane being collided are read again from L1/L2 (to
-// keep the register count down).  Each population crosses DRAM once per step in
-// each direction.
+// One launch per time step: each block owns a 32 x 8 column of the x-y plane and
+// marches through a chunk of z-planes.  The populations that a plane's nodes and
+// their one-node ring pull (pull streaming, supplement Eq. 2) arrive in shared
+// memory by asynchronous copies, two planes ahead; each thread turns its nodes'
+// 19 into the rest population and the nine opposite pairs' sums and differences,
+// keeps those in registers and puts the density into a three-plane ring buffer; the
+// collision of plane z runs once the density of plane z + 1 is there, so the force
+// stencil (Eq. 12) of every node reads its 18 neighbours' densities from shared
+// memory.  Each population crosses DRAM once per step in each direction.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include "lbm.h"
+#include "lbm_tma.cuh"
 
 namespace {
 
@@ -35,13 +34,12 @@ __constant__ int cEX[Q] = {0, 1, -1, 0, 0, 0, 0, 1, -1, 1, -1, 1, -1, 1, -1, 0, 
 __constant__ int cEY[Q] = {0, 0, 0, 1, -1, 0, 0, 1, -1, -1, 1, 0, 0, 0, 0, 1, -1, 1, -1};
 __constant__ int cEZ[Q] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
 
-constexpr int TX = 32, TY = 4, TZ = 32;  // TZ: the longest z-chunk (see chunk_planes)
+constexpr int TX = 32, TY = 8;  // tile of a block in x and y
 constexpr int HX = TX + 2, HY = TY + 2;
-constexpr int kRing = 2 * HX + 2 * TY;  // ring slots of one density plane (76)
-static_assert(kRing <= TX * TY, "every ring slot needs a thread of the block");
+constexpr int kRing = 2 * HX + 2 * TY;  // ring slots of one density plane (84)
 constexpr double kSEps3 = 1.75;
 
-// Collision constants (host: make_c3).
+// Collision constants of the initial state and of k_d3_pull (host: make_c3).
 template <typename T>
 struct C3 {
   int eos;
@@ -64,6 +62,513 @@ __device__ __forceinline__ T p_eos(const C3<T>& c, T rho) {
   return c.lam_RT * rho * z - c.lam_a * rho * rho;
 }
 
+// Velocity components of plane i (folded to constants in unrolled loops).
+__host__ __device__ constexpr int ex3(int i) {
+  return i == 1 || i == 7 || i == 9 || i == 11 || i == 13 ? 1 : (i == 2 || i == 8 || i == 10 || i == 12 || i == 14 ? -1 : 0);
+}
+__host__ __device__ constexpr int ey3(int i) {
+  return i == 3 || i == 7 || i == 10 || i == 15 || i == 17 ? 1
+                                                           : (i == 4 || i == 8 || i == 9 || i == 16 || i == 18 ? -1 : 0);
+}
+__host__ __device__ constexpr int ez3(int i) {
+  return i == 5 || i == 11 || i == 14 || i == 15 || i == 18 ? 1
+                                                            : (i == 6 || i == 12 || i == 13 || i == 16 || i == 17 ? -1 : 0);
+}
+constexpr bool same_velocities() {
+  for (int i = 0; i < Q; ++i)
+    if (ex3(i) != kEX[i] || ey3(i) != kEY[i] || ez3(i) != kEZ[i]) return false;
+  return true;
+}
+static_assert(same_velocities(), "ex3, ey3, ez3 are kEX, kEY, kEZ");
+
+// Value types of the step: r64 (one FP64 node) and f2 (two FP32 nodes per packed
+// instruction); both round every operation as written.
+using lbm::f2;
+using lbm::fmav;
+using lbm::r64;
+
+__device__ __forceinline__ f2 operator-(f2 a) { return f2{make_float2(-a.v.x, -a.v.y)}; }
+
+template <typename V>
+struct Val;
+template <>
+struct Val<f2> {
+  using real = float;
+  static constexpr int lanes = 2;
+  __device__ static f2 pack(const float (&a)[2]) { return f2{make_float2(a[0], a[1])}; }
+  __device__ static float get(f2 v, int k) { return k ? v.v.y : v.v.x; }
+  // Reciprocal: the hardware's approximation (1 ulp) and one Newton step r (2 - x r).
+  __device__ static f2 rcp(f2 x) {
+    const f2 r = lbm::rcp(x);
+    const f2 one{make_float2(1.f, 1.f)};
+    return fmav(r, fmav(-x, r, one), r);
+  }
+  static f2 make(double v) { return f2{make_float2(float(v), float(v))}; }
+};
+template <>
+struct Val<r64> {
+  using real = double;
+  static constexpr int lanes = 1;
+  __device__ static r64 pack(const double (&a)[1]) { return r64{a[0]}; }
+  __device__ static double get(r64 v, int) { return v.v; }
+  __device__ static r64 rcp(r64 x) { return r64{lbm::rcp_fp64(x.v)}; }
+  static r64 make(double v) { return r64{v}; }
+};
+template <typename T>
+struct ValOf;
+template <>
+struct ValOf<float> {
+  using V = f2;
+};
+template <>
+struct ValOf<double> {
+  using V = r64;
+};
+
+// Collision constants (host: make_cv3).  The stencil sums arrive as 12 s.
+template <typename V>
+struct CV3 {
+  int eos;
+  V rho_ref, nbq;                // rho_ref; -b (vdW) or -b / 4 (Carnahan-Starling)
+  V lam_RT3, cA;                 // 3 lam R T, 3 G2 / 2 - 3 lam a
+  V G2s, gq;                     // G2 / 12, G2 / 1728
+  V se, kse, hq;                 // s_e, k s_eps om_e / 19, h s_q om_e 5 / 57 (om_e = s_e / 2 - 1)
+  V ceta, seps_a;                // -(beta_2 + 11 / 2), 2 s_eps / 21
+  V sp3, spi3, bq2, bq23, nbq23;  // s_p / 3, s_pi / 3, 10 bq / 3, 10 bq / 9, its negative (bq = b s_q om_p)
+  V nsp, nbq5;                   // -s_p, -5 bq / 3
+  V sq6, om8;                    // s_q / 6, (1 - s_m) / 8
+  V one, two, three, half, quarter, nquarter, eighth, n2, n3, n4, nhalf;
+  V third, nthird, sixth, n12, twelfth, i24, n2h, n5h, n10h, c1375, c1121;
+};
+
+// Post-collision populations of one node (two for V = f2) from the rest population f0,
+// the pairs' sums s and differences d (plane 2P + 1 plus / minus plane 2P + 2), the
+// density deviation delta = rho - rho_ref and 12 times the force stencil.  All are
+// deviations from w_i rho_ref.  The collision is mbar = m + F_m - S (m - m_eq + F_m / 2
+// - Q_m) with the 3-D S.  Its even part is worked in the variables
+//   a = sum of the axis pairs, T = sum_i |c_i|^2 f_i, Xa = 3 s_0 - a, Xe, Wa, We (the
+//   axis and edge parts of 3p_xx and p_ww), p_xy, p_xz, p_yz,
+// in which the inverse transform is a few additions, and its odd part in d_a, j_a, m_a.
+// With k = J - F (J = rho u): m - m_eq + F_m / 2 is T - delta - eta - k.u (row e),
+// p - (k u) for the second-order rows, and (5 / 3)(j - 3 d) for q.  About 290 operations
+// a node against 364 when every moment was formed (FP64 instructions, measured).
+template <typename V>
+__device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9], const V (&d)[9], V delta, V sx, V sy,
+                                         V sz, V (&o)[Q]) {
+  const V a = s[0] + (s[1] + s[2]);
+  const V E12 = s[3] + s[4], E13 = s[5] + s[6], E23 = s[7] + s[8];
+  const V Ed = E12 + E13 + E23;
+  const V Tr = fmav(c.two, Ed, a);
+  const V Xa = fmav(c.three, s[0], -a), Xe = fmav(c.n3, E23, Ed);
+  const V Wa = s[1] - s[2], We = E12 - E13;
+  const V pxy = s[3] - s[4], pxz = s[5] - s[6], pyz = s[7] - s[8];
+  const V D12p = d[3] + d[4], D12m = d[3] - d[4], D13p = d[5] + d[6], D13m = d[5] - d[6];
+  const V D23p = d[7] + d[8], D23m = d[7] - d[8];
+  const V jx = d[0] + (D12p + D13p), jy = d[1] + (D12m + D23p), jz = d[2] + (D13m + D23m);
+
+  // EOS: p_LBE = p_EOS + G^2 rho^2 / 2 (Eq. 18), eta = 3 p_LBE - rho (Eq. 9).
+  const V rho = delta + c.rho_ref;
+  V ir, p3;  // 1 / rho, 3 p_LBE
+  if (c.eos == LB_EOS_VDW) {
+    const V om = fmav(c.nbq, rho, c.one);
+    const V r = Val<V>::rcp(rho * om);
+    ir = r * om;
+    p3 = rho * fmav(c.cA, rho, c.lam_RT3 * (r * rho));
+  } else {
+    const V om = fmav(c.nbq, rho, c.one), t = c.one - om;
+    const V r = Val<V>::rcp(rho * om);
+    const V io = r * rho;
+    ir = r * om;
+    const V z = fmav(t * t, om, c.one + t) * (io * io * io);  // (1 + t + t^2 - t^3) / (1 - t)^3
+    p3 = rho * fmav(c.lam_RT3, z, c.cA * rho);
+  }
+  const V eta = p3 - rho;
+
+  // Force (Eq. 12), velocity (Eq. 5) and their products.
+  const V G2r = c.G2s * rho;
+  const V Fx = G2r * sx, Fy = G2r * sy, Fz = G2r * sz;
+  const V Jx = fmav(c.half, Fx, jx), Jy = fmav(c.half, Fy, jy), Jz = fmav(c.half, Fz, jz);
+  const V ux = Jx * ir, uy = Jy * ir, uz = Jz * ir;
+  const V X = (Jx - Fx) * ux, Y = (Jy - Fy) * uy, Z = (Jz - Fz) * uz;
+  const V W = X + (Y + Z);
+  const V FX = Fx * ux, FY = Fy * uy, FZ = Fz * uz;
+  const V Fu = FX + (FY + FZ);
+  const V FDxx = fmav(c.three, FX, -Fu), FDww = FY - FZ;
+  // Q_m (Eq. 14 in 3-D, F~ = G s) joins the second-order equilibria: X' = k_x u_x + G^2 s_x^2 / 12.
+  const V gx = c.gq * sx, gy = c.gq * sy, gz = c.gq * sz;
+  const V X1 = fmav(gx, sx, X), Y1 = fmav(gy, sy, Y), Z1 = fmav(gz, sz, Z);
+  const V W1 = X1 + (Y1 + Z1);
+  const V dW = W1 - W;  // G^2 s.s / 12
+
+  // q rows: G_q = (5 / 3) g.
+  const V hx = fmav(c.n3, d[0], jx), hy = fmav(c.n3, d[1], jy), hz = fmav(c.n3, d[2], jz);
+  const V bX = ux * hx, bY = uy * hy, bZ = uz * hz;
+  const V uG = bX + (bY + bZ);
+  // e and eps rows.
+  const V gE = (Tr + c.rho_ref) - (p3 + W);  // T - delta - eta - k.u, delta + eta = 3 p_LBE - rho_ref
+  V ge = fmav(c.n5h, gE, c.ceta * eta);
+  ge = fmav(c.n10h, fmav(c.nthird, delta, a), ge);
+  ge = fmav(c.c1375, dW, ge);
+  const V R = fmav(c.se, fmav(c.n2h, dW, gE), fmav(c.kse, ge, c.hq * uG));
+  const V Ts = fmav(c.two, Fu, Tr) - R;
+  const V as = fmav(c.seps_a, ge, fmav(c.c1121, R, a));
+  // 3p_xx, 3pi_xx, p_ww, pi_ww rows.
+  const V Hxx = fmav(c.three, X1, -W1), Hww = Y1 - Z1;
+  const V Ax = fmav(c.sp3, (Xa + Xe) - Hxx, fmav(c.bq2, bX, c.nbq23 * uG));
+  const V Ix = c.spi3 * fmav(c.half, Hxx, fmav(c.n2, Xa, Xe));
+  const V Xas = (Xa + FDxx) - (Ax - Ix), Xes = (Xe + FDxx) - (Ax + Ax + Ix);
+  const V Aw = fmav(c.sp3, (Wa + We) - Hww, c.bq23 * (bY - bZ));
+  const V Iw = c.spi3 * fmav(c.half, Hww, fmav(c.n2, Wa, We));
+  const V Was = (Wa + FDww) - (Aw - Iw), Wes = (We + FDww) - (Aw + Aw + Iw);
+  // Off-diagonal rows.
+  auto off = [&](V p, V F1, V F2, V J1, V u1, V u2, V g1, V s2, V h1, V h2) {
+    const V Fc = fmav(F1, u2, F2 * u1);
+    const V H = fmav(g1, s2, fmav(c.nhalf, Fc, J1 * u2));
+    return fmav(c.nbq5, fmav(u2, h1, u1 * h2), fmav(c.nsp, p - H, p + Fc));
+  };
+  const V xy = off(pxy, Fx, Fy, Jx, ux, uy, gx, sy, hx, hy);
+  const V xz = off(pxz, Fx, Fz, Jx, ux, uz, gx, sz, hx, hz);
+  const V yz = off(pyz, Fy, Fz, Jy, uy, uz, gy, sz, hy, hz);
+  // Odd part: half differences of the axis pairs, and J of the edges from momentum
+  // conservation (2 od + 8 J = j + F).
+  const V ox = fmav(c.sq6, hx, fmav(c.sixth, Fx, c.half * d[0]));
+  const V oy = fmav(c.sq6, hy, fmav(c.sixth, Fy, c.half * d[1]));
+  const V oz = fmav(c.sq6, hz, fmav(c.sixth, Fz, c.half * d[2]));
+  const V JX = fmav(c.nquarter, ox, c.eighth * (jx + Fx));
+  const V JY = fmav(c.nquarter, oy, c.eighth * (jy + Fy));
+  const V JZ = fmav(c.nquarter, oz, c.eighth * (jz + Fz));
+  const V mx = c.om8 * (D12p - D13p), my = c.om8 * (D23p - D12m), mz = c.om8 * (D13m - D23m);
+
+  // Inverse transform.  o[0] takes what the other populations' even parts leave of the
+  // mass, so that the rounding of their constants does not shift it step by step (200
+  // FP32 steps of 64^3: 3e-6 off 64 bits with o[0] from T and a, 5e-7 with this).
+  const V a6 = c.sixth * as;
+  const V ev0 = fmav(c.sixth, Xas, a6), et = fmav(c.n12, Xas, a6);
+  const V ev1 = fmav(c.quarter, Was, et), ev2 = fmav(c.nquarter, Was, et);
+  o[1] = ev0 + ox, o[2] = ev0 - ox;
+  o[3] = ev1 + oy, o[4] = ev1 - oy;
+  o[5] = ev2 + oz, o[6] = ev2 - oz;
+  const V ce = c.i24 * (Ts - as);
+  const V cx = fmav(c.i24, Xes, ce), eyz = fmav(c.n12, Xes, ce);
+  o[0] = fmav(c.n4, fmav(c.two, cx, eyz), fmav(c.n2, fmav(c.two, et, ev0), delta));
+  const V w8 = c.eighth * Wes;
+  const V exy = cx + w8, exz = cx - w8;
+  auto edge = [&](V e, V p, V odp, V odm, V& o1, V& o2, V& o3, V& o4) {
+    const V ep = fmav(c.quarter, p, e), em = fmav(c.nquarter, p, e);
+    o1 = ep + odp, o2 = ep - odp;
+    o3 = em + odm, o4 = em - odm;
+  };
+  edge(exy, xy, (JX + JY) + (mx - my), (JX - JY) + (mx + my), o[7], o[8], o[9], o[10]);
+  edge(exz, xz, (JX + JZ) - (mx - mz), (JX - JZ) - (mx + mz), o[11], o[12], o[13], o[14]);
+  edge(eyz, yz, (JY + JZ) + (my - mz), (JY - JZ) + (my + mz), o[15], o[16], o[17], o[18]);
+}
+
+// 12 times the force stencil sum_i omega_i rho(x + e_i) e_i (Eq. 12) from the density
+// planes of z - 1 (slot a), z (b) and z + 1 (e); at(slot, dy, dx): density of a neighbour.
+template <typename V, typename At>
+__device__ __forceinline__ void stencil3(const CV3<V>& c, const At& at, int a, int b, int e, V& sx, V& sy, V& sz) {
+  const V u1 = at(b, 1, 1) - at(b, -1, -1), v1 = at(b, -1, 1) - at(b, 1, -1);
+  const V u2 = at(e, 0, 1) - at(a, 0, -1), v2 = at(a, 0, 1) - at(e, 0, -1);
+  const V u3 = at(e, 1, 0) - at(a, -1, 0), v3 = at(a, 1, 0) - at(e, -1, 0);
+  sx = fmav(c.two, at(b, 0, 1) - at(b, 0, -1), (u1 + v1) + (u2 + v2));
+  sy = fmav(c.two, at(b, 1, 0) - at(b, -1, 0), (u1 - v1) + (u3 + v3));
+  sz = fmav(c.two, at(e, 0, 0) - at(a, 0, 0), (u2 - v2) + (u3 - v3));
+}
+
+// Window of one plane of a tile of tw x th nodes: for population i the cells that the
+// pulls of the tile and of its ring read, th + 2 rows (window row r holds lattice row
+// y0 - 1 - e_iy + r) of tw columns and a 16-byte run at each side (window column q =
+// lattice column x0 - XO + q).  FP32 tiles are 32 x 8; FP64 tiles are chosen to fill the
+// SMs (tile_plan), up to the sizes below.
+template <typename T>
+struct Win3 {
+  static constexpr int run = 16 / int(sizeof(T));  // elements of a 16-byte run
+  static constexpr int xo = run;
+  static constexpr bool tensor = sizeof(T) == 4;    // tensor copies (FP32)
+  static constexpr bool fixed = sizeof(T) == 4;     // 32 x 8 tiles
+  static constexpr int cols = TX + 2 * run, rows = HY;
+  static constexpr int cells = fixed ? cols * rows : 416;   // at most, of a window
+  static constexpr int ring_cells = fixed ? HX * HY : 400;  // at most, of a density plane
+  static constexpr int plane = (cells * int(sizeof(T)) + 127) / 128 * 128 / int(sizeof(T));
+  static constexpr int threads = TX * TY / Val<typename ValOf<T>::V>::lanes;
+  static constexpr int stages = 2;
+  static constexpr unsigned smem = unsigned(stages) * Q * plane * sizeof(T) + 128;
+  static_assert(rows * cols / run <= threads && kRing <= threads, "one thread per run and per ring slot");
+};
+static_assert(Win3<float>::plane * 4 % 128 == 0, "a tensor copy's destination is on a 128-byte boundary");
+
+__device__ __forceinline__ int wrap(int a, int n) {
+  a %= n;
+  return a < 0 ? a + n : a;
+}
+
+// Resident blocks per SM: two for FP32 (128 threads of two nodes, up to 255 registers:
+// at three blocks the 168 registers spill and the step is 10% slower), one for FP64
+// (256 threads; its pipe is busy with two warps per scheduler).
+template <typename T>
+constexpr int d3_blocks() {
+  return sizeof(T) == 8 ? 1 : 2;
+}
+
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int w,
+                                            unsigned long long* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+      ::"r"(lbm::smem_addr(dst)), "l"(reinterpret_cast<unsigned long long>(map)), "r"(x), "r"(y), "r"(z), "r"(w),
+      "r"(lbm::smem_addr(bar))
+      : "memory");
+}
+
+// Whether the windows of the tile at (x0, y0) arrive by tensor copies: nineteen a plane
+// (box 40 x 10 of the map (x, y, z, plane)), issued by thread 0 and completing on the
+// stage's mbarrier.  Tiles at the lattice's edge in x or y take 16-byte copies by every
+// thread instead, periodic in every coordinate: the wrapped part as boxes of one 16-byte
+// run was much slower (a 64^3 step, all edge tiles in x, 21 us against 13), and nineteen
+// issuing lanes in place of one thread cost 7%.
+template <typename T>
+__host__ __device__ __forceinline__ bool tensor_tile(int x0, int y0, int nx, int ny) {
+  using W = Win3<T>;
+  return x0 >= W::xo && x0 + TX + W::run <= nx && y0 >= 2 && y0 + TY + 2 <= ny;
+}
+
+// The fused step.  Grid (ceil(nx/tw), ceil(ny/th), ceil(nz/tz)); each block marches a
+// chunk of tz planes (tile_plan picks the three).  VEC: rows of a multiple of 16 bytes; FP32
+// steps then have maps.  err is set by a bounded wait that gave up.
+// have_map: the map is that of fin (else every tile is filled by runs).
+// Iteration p: the window of plane p has arrived; its densities are formed and its
+// populations kept; its buffer is handed to plane p + 2 (plane p + 1 is in flight); plane
+// p - 1, kept from the iteration before, is collided.  Threads of ragged tiles that lie
+// outside the lattice fill their density slot with the wrapped node's and store nothing.
+//
+// FP32 256^3: 529 us a step with the populations pulled into registers (k_d3_pull), 461 to
+// 469 here.  What bounds it: the traffic between L2 and the SMs, 1.56 times the
+// algorithmic reads because of the windows' halo.  Steps that moved the same windows and
+// skipped the collision ran at 34.8 GLUPS with 16-byte copies by the threads whatever the
+// number of blocks and stages, at 38.6 without the halo, and at 39.1 with tensor copies.
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(Win3<T>::threads, d3_blocks<T>())
+    k_d3_step(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, int nz, int tw_, int th_, int tz,
+              const CV3<typename ValOf<T>::V> c, const __grid_constant__ CUtensorMap map, int have_map, int* __restrict__ err) {
+  using V = typename ValOf<T>::V;
+  using W = Win3<T>;
+  constexpr int L = Val<V>::lanes;
+  constexpr bool kTensor = W::tensor && VEC;
+  extern __shared__ __align__(128) unsigned char dyn[];
+  T* win = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
+  __shared__ T rho[3][W::ring_cells];
+  __shared__ __align__(8) unsigned long long bar[W::stages];
+  __shared__ int gave_up;
+  const int tw = W::fixed ? TX : tw_, th = W::fixed ? TY : th_;
+  const int hx = tw + 2, cols = tw + 2 * W::run, runs = cols / W::run;  // pitches of a density plane and a window
+  const int tid = threadIdx.x, tx = tid % tw, ty = tid / tw;
+  const bool node = W::fixed || tid < tw * th;
+  const int x0 = blockIdx.x * tw, y0 = blockIdx.y * th, z0 = blockIdx.z * tz;
+  const int z1 = min(z0 + tz, nz);
+  const size_t N = size_t(nx) * ny * nz;
+  const bool tensor = kTensor && have_map && tensor_tile<T>(x0, y0, nx, ny);
+  if constexpr (kTensor) {
+    if (tid == 0) {
+      gave_up = 0;
+      for (int g = 0; g < W::stages; ++g) lbm::mbar_init(&bar[g], 1);
+    }
+    __syncthreads();
+  }
+
+  // Runs: thread j fills run j mod runs of window row j / runs, all planes.
+  const int cr = tid / runs, cq = (tid - cr * runs) * W::run;
+  const bool copier = tid < (th + 2) * runs;
+  int row[3], col[VEC ? 1 : W::run];
+#pragma unroll
+  for (int e = 0; e < 3; ++e) row[e] = wrap(y0 - e + cr, ny) * nx;  // e_iy + 1
+#pragma unroll
+  for (int q = 0; q < (VEC ? 1 : W::run); ++q) col[q] = wrap(x0 - W::xo + cq + q, nx);
+  auto issue = [&](int zraw, int buf) {
+    const int z = zraw < 0 ? zraw + nz : (zraw >= nz ? zraw - nz : zraw);
+    const int zd = z == 0 ? nz - 1 : z - 1, zu = z == nz - 1 ? 0 : z + 1;
+    T* stage = win + buf * Q * W::plane;
+    if constexpr (kTensor) {
+      if (tensor) {
+        if (tid == 0 && zraw <= z1) {
+          lbm::fence_proxy_async();
+          lbm::mbar_expect_tx(&bar[buf], unsigned(Q * W::rows * W::cols * sizeof(T)));
+#pragma unroll
+          for (int i = 0; i < Q; ++i)
+            tma_load_4d(stage + i * W::plane, &map, x0 - W::xo, y0 - 1 - ey3(i),
+                        ez3(i) == 0 ? z : (ez3(i) > 0 ? zd : zu), i, &bar[buf]);
+        }
+        return;
+      }
+    }
+    if (copier && zraw <= z1) {
+      int zo[3];  // e_iz + 1: plane z - e_iz
+      zo[0] = zu * ny * nx;
+      zo[1] = z * ny * nx;
+      zo[2] = zd * ny * nx;
+      T* dst = stage + (cr * cols + cq);
+      const T* base = fin;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const T* src = base + (zo[ez3(i) + 1] + row[ey3(i) + 1]);
+        if constexpr (VEC) {
+          lbm::cp_async16(dst + i * W::plane, src + col[0]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < W::run; ++q) lbm::cp_async_elem(dst + i * W::plane + q, src + col[q]);
+        }
+        base += N;
+      }
+    }
+    lbm::cp_async_commit();
+  };
+
+  // Nodes of this thread: (tx, ty) and, for FP32, (tx, ty + 4).
+  const int x = x0 + tx;
+  constexpr int kStep = TY / L;
+  // Ring slot of this thread: lower row, upper row, left and right columns.
+  const bool ring = tid < 2 * hx + 2 * th;
+  int hsx = 0, hsy = 0;
+  if (tid < hx) {
+    hsx = tid;
+  } else if (tid < 2 * hx) {
+    hsx = tid - hx;
+    hsy = th + 1;
+  } else if (ring) {
+    const int r = tid - 2 * hx;
+    hsx = r < th ? 0 : tw + 1;
+    hsy = 1 + (r < th ? r : r - th);
+  }
+  // This thread's cells: of its first node in a window and in a density plane, of its ring slot.
+  const int own = (ty + 1) * cols + tx + W::xo, own_rho = (ty + 1) * hx + tx + 1;
+  const int ring_own = hsy * cols + hsx - 1 + W::xo, ring_rho = hsy * hx + hsx;
+  struct Node {
+    V f0, s[9], d[9];
+  };
+  // Populations of the plane staged in buf into n, and the densities of tile and ring
+  // into slot.
+  auto take = [&](int buf, int slot, Node& n) {
+    const T* w = win + buf * Q * W::plane;
+    auto pull = [&](int i) {
+      T v[L];
+#pragma unroll
+      for (int k = 0; k < L; ++k) v[k] = w[i * W::plane + own + k * kStep * cols - ex3(i)];
+      return Val<V>::pack(v);
+    };
+    if (node) {
+      n.f0 = pull(0);
+      V sum = n.f0;
+#pragma unroll
+      for (int P = 0; P < 9; ++P) {
+        const V p = pull(2 * P + 1), m = pull(2 * P + 2);
+        n.s[P] = p + m;
+        n.d[P] = p - m;
+        sum = sum + n.s[P];
+      }
+#pragma unroll
+      for (int k = 0; k < L; ++k) rho[slot][own_rho + k * kStep * hx] = Val<V>::get(sum, k);
+    }
+    if (ring) {
+      const T* r = w + ring_own;
+      T a = r[0];
+#pragma unroll
+      for (int P = 0; P < 9; ++P)
+        a += r[(2 * P + 1) * W::plane - ex3(2 * P + 1)] + r[(2 * P + 2) * W::plane - ex3(2 * P + 2)];
+      rho[slot][ring_rho] = a;
+    }
+  };
+  auto collide = [&](int z, int sp, int sc, int sn, const Node& n) {
+    if (!node) return;
+    auto at = [&](int slot, int dy, int dx) {
+      T v[L];
+#pragma unroll
+      for (int k = 0; k < L; ++k) v[k] = rho[slot][own_rho + k * kStep * hx + dy * hx + dx];
+      return Val<V>::pack(v);
+    };
+    V sx, sy, sz;
+    stencil3(c, at, sp, sc, sn, sx, sy, sz);
+    V o[Q];
+    collide3(c, n.f0, n.s, n.d, at(sc, 0, 0), sx, sy, sz, o);
+#pragma unroll
+    for (int k = 0; k < L; ++k) {
+      const int y = y0 + ty + k * kStep;
+      if (x < nx && y < ny) {
+        T* p = fout + ((z * ny + y) * nx + x);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+          *p = Val<V>::get(o[i], k);
+          p += N;
+        }
+      }
+    }
+  };
+
+  // S windows in flight: group g holds plane z0 - 1 + g and lands in buffer g mod S.
+  constexpr int S = W::stages;
+  int buf = 0;
+  unsigned phase = 0;  // bit g: parity of the next phase of bar[g]
+  // Waits for the oldest window; false (for the whole block) if that gave up, with no
+  // copy of this block left in flight unless its bounded waits gave up as well.  (A flag
+  // in shared memory: a barrier that also reduces a predicate cost 3% of the step.)
+  auto arrive = [&]() {
+    if constexpr (kTensor) {
+      if (tensor) {
+        if (!lbm::mbar_wait(&bar[buf], phase >> buf & 1u)) gave_up = 1;
+        phase ^= 1u << buf;
+      }
+    }
+    if (!tensor) asm volatile("cp.async.wait_group %0;" ::"n"(S - 1) : "memory");
+    __syncthreads();
+    if constexpr (kTensor) {
+      if (gave_up) {
+        if (tid == 0) {
+          atomicExch(err, 1);
+          for (int g = 0; g < S; ++g) lbm::mbar_wait(&bar[g], (g == buf ? phase ^ (1u << buf) : phase) >> g & 1u);
+        }
+        __syncthreads();
+        return false;
+      }
+    }
+    return true;
+  };
+  auto release = [&](int zraw) {  // its buffer, for plane zraw
+    __syncthreads();
+    issue(zraw, buf);
+    buf = buf == S - 1 ? 0 : buf + 1;
+  };
+  // Plane p: taken into next; the plane before it, cur, is collided (from z0 on).
+  Node A, B;
+  int sp = 1, sc = 2, sn = 0;
+  auto plane = [&](int p, const Node& cur, Node& next) {
+    if (!arrive()) return false;
+    take(buf, sn, next);
+    release(p + S);
+    if (p > z0) collide(p - 1, sp, sc, sn, cur);
+    const int t = sp;
+    sp = sc;
+    sc = sn;
+    sn = t;
+    return true;
+  };
+#pragma unroll 1
+  for (int g = 0; g < S; ++g) issue(z0 - 1 + g, g);
+#pragma unroll 1
+  for (int p = z0 - 1; p <= z1; p += 2) {
+    if (!plane(p, A, B)) return;
+    if (p < z1 && !plane(p + 1, B, A)) return;
+  }
+  lbm::cp_async_wait_all();
+}
+
+// ---------------------------------------------------------------------------
+// FP32 lattices whose rows are not a multiple of 16 bytes.  Filling windows element by
+// element is slower than pulling the populations straight into registers (250 x 130 x 77:
+// 131 us a step against 89), and so is this kernel with collide3 (104 us: its loads then
+// wait).  32 x 4 tiles, one node per thread, z-marching chunks of up to 32 planes; a
+// software pipeline in registers: while plane z collides, the pulls of plane z + 2 are in
+// flight, plane z + 1 is summed and held, plane z is in fc (3 blocks per SM).
+constexpr int kPullTY = 4, kPullTZ = 32, kPullHY = kPullTY + 2;
+constexpr int kPullRing = 2 * HX + 2 * kPullTY;
+static_assert(kPullRing <= TX * kPullTY, "every ring slot needs a thread of the block");
+
 // Post-collision populations o (deviations from w_i rho_ref) of one node from
 // its post-streaming deviations f, its density deviation delta = rho - rho_ref
 // and the force stencil sum s = sum_i omega_i rho(x + e_i) e_i.  Moments are the
@@ -72,7 +577,7 @@ __device__ __forceinline__ T p_eos(const C3<T>& c, T rho) {
 // mbar = m + F_m - S (m - m_eq + F_m/2 - Q_m) with the 3-D S, and the inverse
 // uses M^-1 = M^T diag(1 / |row|^2).
 template <typename T>
-__device__ __forceinline__ void collide3(const C3<T>& c, const T* f, T delta, T sx, T sy, T sz, T* o) {
+__device__ __forceinline__ void collide3_moments(const C3<T>& c, const T* f, T delta, T sx, T sy, T sz, T* o) {
   T s[9], d[9];
 #pragma unroll
   for (int P = 0; P < 9; ++P) {
@@ -257,10 +762,6 @@ __device__ __forceinline__ T sum19(const T* v) {
   return a;
 }
 
-__device__ __forceinline__ int wrap(int a, int n) {
-  a %= n;
-  return a < 0 ? a + n : a;
-}
 __device__ __forceinline__ int dec(int a, int n) { return a == 0 ? n - 1 : a - 1; }
 __device__ __forceinline__ int inc(int a, int n) { return a == n - 1 ? 0 : a + 1; }
 
@@ -280,26 +781,19 @@ __device__ __forceinline__ void stencil_collide_store(const C3<T>& c, const T (*
                 T(1.0 / 12.0) * ((e[ly][lx + 1] - a[ly][lx - 1]) + (e[ly][lx - 1] - a[ly][lx + 1]) +
                                  (e[ly + 1][lx] - a[ly - 1][lx]) + (e[ly - 1][lx] - a[ly + 1][lx]));
   T o[Q];
-  collide3(c, fc, b[ly][lx], sxv, syv, szv, o);
+  collide3_moments(c, fc, b[ly][lx], sxv, syv, szv, o);
 #pragma unroll
   for (int i = 0; i < Q; ++i) fout[i * N + idx] = o[i];
 }
 
-// The fused step.  Grid (ceil(nx/32), ceil(ny/4), ceil(nz/tz)), block (32, 4); each
-// block marches a chunk of tz <= 32 planes (chunk_planes picks tz).
-// Threads of ragged tiles that lie outside the lattice fill their ring-buffer
-// slot with the density of the wrapped node and do not collide.
-//   KEEP (FP32, 3 blocks per SM, up to 170 registers): software pipeline in
-//   registers; while plane z collides, the pulls of plane z + 2 are in flight,
-//   plane z + 1 is summed and held, plane z is in fc.
-//   !KEEP (FP64, 4 blocks per SM): plane z + 1 is pulled and summed before the
-//   collision of plane z, whose populations are read again (L1 / L2).
-template <typename T, bool KEEP, typename S>
-__global__ void __launch_bounds__(TX* TY, KEEP ? 3 : 4)
-    k_d3_step(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, int nz, int tz, C3<T> c) {
-  __shared__ T pl[3][HY][HX];
+// S: type of the plane offsets (int when 19 nx ny nz < 2^31, else long long).
+template <typename S>
+__global__ void __launch_bounds__(TX* kPullTY, 3)
+    k_d3_pull(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int nz, int tz, C3<float> c) {
+  using T = float;
+  __shared__ T pl[3][kPullHY][HX];
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = blockIdx.z * tz;
+  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * kPullTY, z0 = blockIdx.z * tz;
   const int z1 = min(z0 + tz, nz);
   const S N = S(nx) * ny * nz;
   const int x = x0 + tx, y = y0 + ty;
@@ -307,17 +801,17 @@ __global__ void __launch_bounds__(TX* TY, KEEP ? 3 : 4)
   const int xg = x % nx, yg = y % ny;
   const int xm = dec(xg, nx), xp = inc(xg, nx), ym = dec(yg, ny), yp = inc(yg, ny);
   // Ring slot of this thread (threads 0..75): top row, bottom row, left and right columns.
-  const bool ring = tid < kRing;
+  const bool ring = tid < kPullRing;
   int hsx = 0, hsy = 0;
   if (tid < HX) {
     hsx = tid;
   } else if (tid < 2 * HX) {
     hsx = tid - HX;
-    hsy = HY - 1;
+    hsy = kPullHY - 1;
   } else if (ring) {
     const int r = tid - 2 * HX;
-    hsx = r < TY ? 0 : HX - 1;
-    hsy = 1 + (r < TY ? r : r - TY);
+    hsx = r < kPullTY ? 0 : HX - 1;
+    hsy = 1 + (r < kPullTY ? r : r - kPullTY);
   }
   const int hx = wrap(x0 - 1 + hsx, nx), hy = wrap(y0 - 1 + hsy, ny);
   const int hxm = dec(hx, nx), hxp = inc(hx, nx), hym = dec(hy, ny), hyp = inc(hy, ny);
@@ -338,60 +832,33 @@ __global__ void __launch_bounds__(TX* TY, KEEP ? 3 : 4)
 
   T fc[Q], fn[Q];
   int sp = 0, sc = 1, sn = 2;
-  if constexpr (KEEP) {
-    T fr[Q], gn[Q], gr[Q];
-    pull_node(z0 - 1, fn);
-    if (ring) pull_ring(z0 - 1, fr);
-    put(0, fn, fr);
-    pull_node(z0, fc);
-    if (ring) pull_ring(z0, fr);
-    put(1, fc, fr);
-    pull_node(z0 + 1, fn);
-    if (ring) pull_ring(z0 + 1, fr);
-    for (int z = z0; z < z1; ++z) {
-      put(sn, fn, fr);
-      if (z + 1 < z1) {
-        pull_node(z + 2, gn);
-        if (ring) pull_ring(z + 2, gr);
-      }
-      __syncthreads();
-      if (active) stencil_collide_store(c, pl[sp], pl[sc], pl[sn], ty + 1, tx + 1, fc, fout, N, (z * ny + y) * nx + x);
-      __syncthreads();
-      const int t = sp;
-      sp = sc;
-      sc = sn;
-      sn = t;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        fc[i] = fn[i];
-        fn[i] = gn[i];
-        fr[i] = gr[i];
-      }
+  T fr[Q], gn[Q], gr[Q];
+  pull_node(z0 - 1, fn);
+  if (ring) pull_ring(z0 - 1, fr);
+  put(0, fn, fr);
+  pull_node(z0, fc);
+  if (ring) pull_ring(z0, fr);
+  put(1, fc, fr);
+  pull_node(z0 + 1, fn);
+  if (ring) pull_ring(z0 + 1, fr);
+  for (int z = z0; z < z1; ++z) {
+    put(sn, fn, fr);
+    if (z + 1 < z1) {
+      pull_node(z + 2, gn);
+      if (ring) pull_ring(z + 2, gr);
     }
-  } else {
-    // One array at a time: pull, sum, then the ring slot's pull and sum.
-    auto density = [&](int zraw, int slot) {
-      pull_node(zraw, fn);
-      pl[slot][ty + 1][tx + 1] = sum19(fn);
-      if (ring) {
-        pull_ring(zraw, fn);
-        pl[slot][hsy][hsx] = sum19(fn);
-      }
-    };
-    density(z0 - 1, 0);
-    density(z0, 1);
-    for (int z = z0; z < z1; ++z) {
-      density(z + 1, sn);
-      __syncthreads();
-      if (active) {
-        pull_node(z, fc);
-        stencil_collide_store(c, pl[sp], pl[sc], pl[sn], ty + 1, tx + 1, fc, fout, N, (z * ny + y) * nx + x);
-      }
-      __syncthreads();
-      const int t = sp;
-      sp = sc;
-      sc = sn;
-      sn = t;
+    __syncthreads();
+    if (active) stencil_collide_store(c, pl[sp], pl[sc], pl[sn], ty + 1, tx + 1, fc, fout, N, (z * ny + y) * nx + x);
+    __syncthreads();
+    const int t = sp;
+    sp = sc;
+    sc = sn;
+    sn = t;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      fc[i] = fn[i];
+      fn[i] = gn[i];
+      fr[i] = gr[i];
     }
   }
 }

@@ -319,6 +319,23 @@ bool encode_plane_map(CUtensorMap* map, const void* base, int nx, int ny, int pl
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// 4-D map (x, y, z, plane) of `planes` FP32 volumes of nx x ny x nz, box of cols x rows x
+// 1 x 1.
+bool encode_volume_map(CUtensorMap* map, const void* base, int nx, int ny, int nz, int planes, int cols, int rows) {
+  const EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  if (reinterpret_cast<uintptr_t>(base) % 16 != 0 || (size_t(nx) * 4) % 16 != 0 || nx < cols || ny < rows)
+    return false;
+  const cuuint64_t row = cuuint64_t(nx) * 4;
+  const cuuint64_t dims[4] = {cuuint64_t(nx), cuuint64_t(ny), cuuint64_t(nz), cuuint64_t(planes)};
+  const cuuint64_t strides[3] = {row, row * ny, row * ny * nz};
+  const cuuint32_t box[4] = {cuuint32_t(cols), cuuint32_t(rows), 1, 1};
+  const cuuint32_t estride[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void*>(base), dims, strides, box, estride,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace lbm
 
 namespace {

@@ -73,6 +73,9 @@ bool encode_population_map(CUtensorMap* map, void* base, int nx, int ny, int sx,
 // 3-D map (x, y, plane) of `planes` FP32 planes of nx x ny, box cols x rows x 1
 // (lbm_capi.cu); false if the buffer does not allow one.
 bool encode_plane_map(CUtensorMap* map, const void* base, int nx, int ny, int planes, int cols, int rows);
+// 4-D map (x, y, z, plane) of `planes` FP32 volumes of nx x ny x nz, box of cols x rows x
+// 1 x 1 (lbm_capi.cu); false if the buffer does not allow one.
+bool encode_volume_map(CUtensorMap* map, const void* base, int nx, int ny, int nz, int planes, int cols, int rows);
 // Cut of a lattice for the resident run; false if it does not fit (lbm_resident.cu).
 bool res_plan(int nx, int ny, int precision, ResPlan* out);
 // Bytes of the exchange buffer (0 when no precision of this size runs resident).
