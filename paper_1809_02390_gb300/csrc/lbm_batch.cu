@@ -725,10 +725,20 @@ int lb_batch_init(lb_batch** out, const lb_params* ps, int n, void* pool_a, void
     std::snprintf(msg, sizeof(msg), "lb_batch_init: %s", cudaGetErrorString(e));
     return bail(LB_ECUDA, msg);
   }
-  b->shape = 0;
-  int mb = 1;
-  if (max_blocks(b, 0, &mb) != LB_OK) return bail(LB_ECUDA, b->err);
-  b->blocks_per_sm = mb;
+  // Launch form until lb_batch_tune or lb_batch_set_config choose one (the results are the
+  // same).  Pools that L2 holds: one block per tile at 80 registers (48 lattices, 0.92 M
+  // nodes: 16.9 us a step, tickets 20.8, the persistent plain-load grid 21.6); larger
+  // ones: tensor copies with tiles by ticket (6.7 M nodes: 96.9 us, one block per tile
+  // 111, the plain-load grid 139).  The line lies at 100 MB of the 129 MB of L2: 1.18 M
+  // nodes (85 MB) 21.5 against 23.7 us, 4.9 M (351 MB) 81.5 against 72.2.
+  b->shape = 1;
+  b->blocks_per_sm = 0;
+  if (b->tma_ok && 2 * off * sizeof(float) > (size_t(100) << 20)) {
+    int mb = 1;
+    if (max_blocks(b, kShapeDyn, &mb) != LB_OK) return bail(LB_ECUDA, b->err);
+    b->shape = kShapeDyn;
+    b->blocks_per_sm = mb;
+  }
   b->steps = 0;
   *out = b;
   return LB_OK;
