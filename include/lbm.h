@@ -171,6 +171,13 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
  * captured into a graph of its own, every step is a plain launch on that stream. */
 int lb_step(lb_handle* h, int64_t nsteps);
 
+/* lb_step, and the states after every `every` >= 1 steps stored one after the other at
+ * `states` (device memory of (nsteps / every) * lb_state_bytes() bytes, in the handle's
+ * layout and storage type; 16-byte aligned for the fastest path): the trajectory an
+ * adjoint needs, without a copy per step.  The same bits as lb_step and lb_get_state in
+ * turn.  Asynchronous. */
+int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states);
+
 /* Device pointer of the buffer holding the current state. */
 void* lb_state(lb_handle* h);
 

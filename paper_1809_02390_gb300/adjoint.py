@@ -72,18 +72,16 @@ def _make_function():
     class _Rollout(torch.autograd.Function):
         @staticmethod
         def forward(ctx, theta, f0, spec, nsteps, checkpoint_every):
-            lat = Lattice(np.full((spec.ny, spec.nx), 0.5 * (spec.rho_g + spec.rho_l)), precision=spec.precision,
-                          rho_ref=spec.rho_ref, **spec.lattice_kwargs(theta.detach().cpu().numpy()))
+            # (The densities only make a valid handle: its state is f0's.)
+            dev = torch.device("cuda", torch.cuda.current_device())
+            rest = torch.full((spec.ny, spec.nx), 0.5 * (spec.rho_g + spec.rho_l), dtype=torch.float64, device=dev)
+            lat = Lattice(rest, precision=spec.precision, rho_ref=spec.rho_ref,
+                          **spec.lattice_kwargs(theta.detach().cpu().numpy()))
             capi.lb_set_state(lat.h, f0.detach().contiguous().data_ptr())
-            checkpoints = [f0.detach().clone()]
-            done = 0
-            while done < nsteps:
-                k = min(checkpoint_every, nsteps - done)
-                lat.step(k)
-                done += k
-                if done < nsteps:
-                    checkpoints.append(lat.state().clone())
+            stored = torch.empty((nsteps // checkpoint_every, *lat.f_a.shape), dtype=lat.dtype, device=dev)
+            capi.lb_step_record(lat.h, nsteps, checkpoint_every, stored.data_ptr())
             out = lat.state().clone()
+            checkpoints = [f0.detach().clone(), *stored[:(nsteps - 1) // checkpoint_every]]
             ctx.save_for_backward(theta)
             ctx.spec, ctx.nsteps, ctx.every = spec, nsteps, checkpoint_every
             ctx.checkpoints = checkpoints
@@ -101,18 +99,20 @@ def _make_function():
             scratch = torch.empty(nscr, dtype=torch.uint8, device=dev)
             dtheta = torch.zeros(3, dtype=torch.float64, device=dev)
             nseg = len(ctx.checkpoints)
+            # The states of one segment after its checkpoint; every segment reuses the
+            # buffer, in stream order.
+            traj = torch.empty((max(min(ctx.every, ctx.nsteps) - 1, 0), *lat.f_a.shape), dtype=lat.dtype, device=dev)
+            size = lat.f_a.numel() * lat.f_a.element_size()
             for seg in range(nseg - 1, -1, -1):
                 start = seg * ctx.every
                 k = min(ctx.every, ctx.nsteps - start)
                 # Recompute the states s^start .. s^(start+k-1) of this segment, then
                 # run the segment's adjoint steps backwards in one call.
-                states = [ctx.checkpoints[seg]]
-                capi.lb_set_state(lat.h, ctx.checkpoints[seg].data_ptr())
-                for _ in range(k - 1):
-                    lat.step(1)
-                    states.append(lat.state().clone())
-                capi.lb_adjoint_steps(lat.h, [t.data_ptr() for t in states], lam.data_ptr(), dtheta.data_ptr(),
-                                      scratch.data_ptr(), nscr)
+                first = ctx.checkpoints[seg].data_ptr()
+                capi.lb_set_state(lat.h, first)
+                capi.lb_step_record(lat.h, max(k - 1, 0), 1, traj.data_ptr())
+                capi.lb_adjoint_steps(lat.h, [first] + [traj.data_ptr() + j * size for j in range(k - 1)],
+                                      lam.data_ptr(), dtheta.data_ptr(), scratch.data_ptr(), nscr)
             dT, dG2, dlam = (float(v) for v in dtheta.cpu())
             Tr, G2, K = (float(v) for v in theta.detach().cpu())
             lam_val = spec.lam_ref * (spec.K_ref / K) ** 2

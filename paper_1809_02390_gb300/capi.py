@@ -57,6 +57,7 @@ SIGNATURES = [
     ("lb_scratch_bytes", ctypes.c_size_t, [_P]),
     ("lb_init", ctypes.c_int, [ctypes.POINTER(_V), _P, _V, _V, _V, ctypes.c_size_t, _V, ctypes.c_int, _V]),
     ("lb_step", ctypes.c_int, [_V, ctypes.c_int64]),
+    ("lb_step_record", ctypes.c_int, [_V, ctypes.c_int64, ctypes.c_int64, _V]),
     ("lb_state", _V, [_V]),
     ("lb_steps_done", ctypes.c_int64, [_V]),
     ("lb_moments", ctypes.c_int, [_V, _V, _V, _V]),
@@ -177,6 +178,10 @@ def lb_init(p: lb_params, f_a: int, f_b: int, scratch: int, scratch_bytes: int, 
 
 def lb_step(h: int, nsteps: int) -> None:
     check(lib().lb_step(h, int(nsteps)), h)
+
+
+def lb_step_record(h: int, nsteps: int, every: int, states: int) -> None:
+    check(lib().lb_step_record(h, int(nsteps), int(every), states), h)
 
 
 def lb_state(h: int) -> int:

@@ -775,7 +775,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
   }
   if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= kResMinSteps && capture == cudaStreamCaptureStatusNone) {
-    LB_CUDA(h, res_run(h, nsteps, nullptr));
+    LB_CUDA(h, res_run(h, nsteps, nullptr, 1));
     return LB_OK;
   }
   if (nsteps >= kStepGraph && !h->graph_off && capture == cudaStreamCaptureStatusNone) {
@@ -805,6 +805,67 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     ++h->steps;
   }
   return LB_OK;
+}
+
+int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
+  if (!h) return fail(nullptr, LB_EINVAL, "null handle");
+  if (nsteps < 0) return fail(h, LB_EINVAL, "nsteps must be >= 0");
+  if (every < 1 || every > INT32_MAX) return fail(h, LB_EINVAL, "every must be in [1, 2^31)");
+  if (nsteps < every) return lb_step(h, nsteps);
+  if (!states) return fail(h, LB_EINVAL, "null state buffer");
+  const size_t bytes = lb_state_bytes(&h->p);
+  char* at = static_cast<char*>(states);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess) {
+    cudaGetLastError();
+    capture = cudaStreamCaptureStatusActive;
+  }
+  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= 2 && capture == cudaStreamCaptureStatusNone) {
+    LB_CUDA(h, res_run(h, nsteps, states, every));
+    return LB_OK;
+  }
+  const bool aligned = reinterpret_cast<uintptr_t>(at) % 16 == 0 && bytes % 16 == 0;
+  if (every == 1 && (aligned || !h->use_tma)) {
+    // Every state is wanted: step from each straight into the next (the handle's buffers
+    // stand aside), and bring the last one home.
+    void* const f[2] = {h->f[0], h->f[1]};
+    const CUtensorMap maps[2] = {h->tmap[0], h->tmap[1]};
+    const int home = h->cur;
+    void* src = h->f[home];
+    CUtensorMap map = h->tmap[home];
+    cudaError_t e = cudaSuccess;
+    bool mapped = true;
+    int64_t done = 0;
+    for (; done < nsteps && e == cudaSuccess && mapped; ++done) {
+      void* dst = at + size_t(done) * bytes;
+      h->f[0] = src;
+      h->f[1] = dst;
+      h->tmap[0] = map;
+      h->cur = 0;
+      launch_one_step(h);
+      e = cudaGetLastError();
+      ++h->steps;
+      src = dst;
+      if (h->use_tma)
+        mapped = encode_population_map(&map, dst, h->p.nx, h->p.ny, h->p.nx, int(elem_bytes(h->p.precision)),
+                                       h->p.layout == LB_LAYOUT_ROWS);
+    }
+    for (int k = 0; k < 2; ++k) {
+      h->f[k] = f[k];
+      h->tmap[k] = maps[k];
+    }
+    h->cur = done & 1 ? 1 - home : home;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h->f[h->cur], src, bytes, cudaMemcpyDeviceToDevice, h->stream);
+    LB_CUDA(h, e);
+    nsteps -= done;
+    at += size_t(done) * bytes;
+  }
+  for (; nsteps >= every; nsteps -= every, at += bytes) {
+    const int rc = lb_step(h, every);
+    if (rc != LB_OK) return rc;
+    LB_CUDA(h, cudaMemcpyAsync(at, h->f[h->cur], bytes, cudaMemcpyDeviceToDevice, h->stream));
+  }
+  return lb_step(h, nsteps);
 }
 
 void* lb_state(lb_handle* h) { return h ? h->f[h->cur] : nullptr; }

@@ -84,8 +84,8 @@ size_t res_mail_bytes(int nx, int ny);
 // (device memory of res_mail_bytes, 16-byte aligned, or null).
 cudaError_t res_configure(lb_handle* h, void* mail);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
-// null): device memory that receives the state after each step, one after the other.
-cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec);
+// null): device memory that receives the states after every `every` (< 2^31) steps.
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every);
 // Device address of lb_reduce_static's static scratch on the current device
 // (looked up once per device, which commits the array there; lbm_static.cu).
 int static_scratch_address(lb_handle* h, void** out);

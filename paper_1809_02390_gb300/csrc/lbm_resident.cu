@@ -107,13 +107,15 @@ cudaError_t res_configure(lb_handle* h, void* mail) {
 namespace {
 
 template <typename V, typename S>
-cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout, void* rec, long long rec_stride,
-                   int nsteps) {
+cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout, void* rec, int rec_first,
+                   int rec_every, int nsteps) {
   const ResPlan& p = h->res;
   ResArgs<S> a{static_cast<const S*>(fin),
                static_cast<S*>(fout),
                static_cast<S*>(rec),
-               rec_stride,
+               9ll * h->p.nx * h->p.ny,
+               rec_first,
+               rec_every,
                static_cast<uint4*>(h->res_mail),
                h->wait_error,
                h->res_epoch,
@@ -138,9 +140,8 @@ cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout,
 // Steps of one launch: a few milliseconds, so that other work on the GPU gets its turn.
 constexpr int64_t kResChunk = 4096;
 
-cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec) {
-  const long long stride = 9ll * h->p.nx * h->p.ny;
-  const size_t elem = h->p.precision == LB_FP64 ? 8 : h->p.precision == LB_FP32 ? 4 : 2;
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
+  int64_t first = every;  // steps until the next recorded state
   while (nsteps > 0) {
     // Never a launch of one step: it could not write its result in place.
     int64_t n = nsteps <= kResChunk ? nsteps : (nsteps == kResChunk + 1 ? kResChunk - 2 : kResChunk);
@@ -153,12 +154,16 @@ cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec) {
     void* out = h->f[n & 1 ? 1 - h->cur : h->cur];
     cudaError_t e;
     switch (h->p.precision) {
-      case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, stride, int(n)); break;
-      case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, stride, int(n)); break;
-      default: e = launch<f2, __half>(h, h->c2, in, out, rec, stride, int(n)); break;
+      case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, int(first), int(every), int(n)); break;
+      case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
+      default: e = launch<f2, __half>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
     }
     if (e != cudaSuccess) return e;
-    if (rec) rec = static_cast<char*>(rec) + size_t(n) * stride * elem;
+    if (rec) {
+      const int64_t states = n >= first ? 1 + (n - first) / every : 0;
+      rec = static_cast<char*>(rec) + size_t(states) * lb_state_bytes(&h->p);
+      first = states ? every - (n - first) % every : first - n;
+    }
     h->res_epoch += unsigned(n);
     h->steps += n;
     if (n & 1) h->cur = 1 - h->cur;

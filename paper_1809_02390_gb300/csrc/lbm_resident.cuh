@@ -114,8 +114,9 @@ template <typename S>
 struct ResArgs {
   const S* fin;        // state the run starts from
   S* fout;             // state after the last step (may be fin: see k_resident)
-  S* rec;              // or null: the state after step s goes to rec + s * rec_stride
-  long long rec_stride;
+  S* rec;              // or null: the states after `rec_first` steps and every rec_every after
+  long long rec_stride;  // go here, rec_stride elements apart
+  int rec_first, rec_every;
   uint4* mail;         // exchange words, two parities
   int* err;
   unsigned epoch;      // step s carries the number epoch + s + 1
@@ -394,6 +395,8 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
   for (int q = inner_begin; q < sl.total; q += T) density(cur, q);  // phase 1a of step 0
 
   constexpr int W = ResTraits<S>::words;
+  S* rec = a.rec;
+  int until = a.rec_first;  // steps until the next recorded state
   for (int s = 0;; ++s) {
     const unsigned number = a.epoch + unsigned(s);
     bool late = false;
@@ -454,6 +457,7 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
     __syncthreads();
     // Phase 2.
     const bool last = s + 1 == a.nsteps;
+    const bool record = rec != nullptr && --until == 0;
     const unsigned seed = sizeof(S) == 2 ? step_seed(a.step0 + unsigned(s)) : 0u;
     if (gated) asm volatile("bar.sync 2, %0;" ::"r"(gate_threads) : "memory");
     for (int q = tid; q < sl.total; q += T) {
@@ -482,7 +486,7 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
 #pragma unroll
         for (int k = 0; k < L; ++k) {
           int gx = 0, gy = 0;
-          if (last || a.rec || sizeof(S) == 2) {
+          if (last || record || sizeof(S) == 2) {
             gy = o[k] / pitch;
             gx = x0 + (o[k] - gy * pitch) - 2;
             gy += y0 - 2;
@@ -499,10 +503,9 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
 #pragma unroll
             for (int i = 0; i < 9; ++i) a.fout[g + i * a.st.ps] = v[i];
           }
-          if (a.rec) {
-            S* p = a.rec + (long long)s * a.rec_stride + g;
+          if (record) {
 #pragma unroll
-            for (int i = 0; i < 9; ++i) p[i * a.st.ps] = v[i];
+            for (int i = 0; i < 9; ++i) rec[g + i * a.st.ps] = v[i];
           }
         }
       }
@@ -518,6 +521,10 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
       }
     }
     if (last) break;
+    if (record) {
+      rec += a.rec_stride;
+      until = a.rec_every;
+    }
     __syncthreads();
     S* t = cur;
     cur = nxt;
