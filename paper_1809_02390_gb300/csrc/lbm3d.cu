@@ -132,15 +132,15 @@ __global__ void __launch_bounds__(256) k_d3_reduce_partial(const T* __restrict__
   if (threadIdx.x < kReduceSlots3) part[blockIdx.x * kReduceSlots3 + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-__global__ void k_d3_reduce_final(const double* __restrict__ part, int blocks, double* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k >= kReduceSlots3) return;
+// (One warp per slot, lanes over the blocks, a fixed order.)
+__global__ void __launch_bounds__(32 * kReduceSlots3)
+    k_d3_reduce_final(const double* __restrict__ part, int blocks, double* __restrict__ out) {
+  const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double a = k == 5 ? INFINITY : (k == 6 ? -INFINITY : 0.0);
-  for (int b = 0; b < blocks; ++b) {
-    const double x = part[b * kReduceSlots3 + k];
-    a = k == 5 ? fmin(a, x) : (k == 6 ? fmax(a, x) : a + x);
-  }
-  out[k] = a;
+  auto fold = [&](double x, double y) { return k == 5 ? fmin(x, y) : (k == 6 ? fmax(x, y) : x + y); };
+  for (int b = lane; b < blocks; b += 32) a = fold(a, part[b * kReduceSlots3 + k]);
+  for (int w = 16; w > 0; w >>= 1) a = fold(a, __shfl_xor_sync(0xffffffffu, a, w));
+  if (lane == 0) out[k] = a;
 }
 
 }  // namespace
@@ -653,7 +653,7 @@ int lb_d3_reduce(lb_d3_handle* h, double out[8]) {
     k_d3_reduce_partial<float><<<blocks, 256, 0, h->stream>>>(static_cast<const float*>(f), N, h->p.rho_ref, mid,
                                                                h->part);
   double* res = h->part + kReduceBlocks3 * kReduceSlots3;
-  k_d3_reduce_final<<<1, 32, 0, h->stream>>>(h->part, blocks, res);
+  k_d3_reduce_final<<<1, 32 * kReduceSlots3, 0, h->stream>>>(h->part, blocks, res);
   cudaError_t e = cudaMemcpyAsync(out, res, kReduceSlots3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return fail3(h, LB_ECUDA, "reduction: %s", cudaGetErrorString(e));

@@ -535,21 +535,19 @@ int run_reduce(lb_handle* h, double out[8]) {
   const double rho_mid = 0.5 * (h->d.rho_g + h->d.rho_l);
   k_reduce_partial<real, store_t><<<h->reduce_blocks, kReduceThreads, 0, h->stream>>>(
       f, rho, nx, ny, h->st, real(h->d.G2), std::isfinite(rho_mid) ? rho_mid : 1e300, partial);
-  k_reduce_final<<<1, 32, 0, h->stream>>>(partial, h->reduce_blocks, dout);
-  double res[kReduceSlots];
-  real probe[2];
+  k_reduce_final<real><<<1, kFoldThreads, 0, h->stream>>>(partial, h->reduce_blocks, rho, size_t(ny / 2) * nx + nx / 2,
+                                                          dout);
+  double got[2 + kReduceSlots];
   LB_CUDA(h, cudaGetLastError());
-  LB_CUDA(h, cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, h->stream));
-  LB_CUDA(h, cudaMemcpyAsync(&probe[0], rho + size_t(ny / 2) * nx + nx / 2, sizeof(real), cudaMemcpyDeviceToHost,
-                             h->stream));
-  LB_CUDA(h, cudaMemcpyAsync(&probe[1], rho, sizeof(real), cudaMemcpyDeviceToHost, h->stream));
+  LB_CUDA(h, cudaMemcpyAsync(got, dout - 2, sizeof(got), cudaMemcpyDeviceToHost, h->stream));
   LB_CUDA(h, cudaStreamSynchronize(h->stream));
+  const double *probe = got, *res = got + 2;
   // p_EOS / c^2 at the two probe nodes, FP64 on the host.
   out[0] = res[0];
   out[1] = res[1];
   out[2] = res[2];
-  out[3] = p_eos_host(h->cd, double(probe[0]));
-  out[4] = p_eos_host(h->cd, double(probe[1]));
+  out[3] = p_eos_host(h->cd, probe[0]);
+  out[4] = p_eos_host(h->cd, probe[1]);
   out[5] = res[3];
   out[6] = res[4];
   out[7] = res[5];

@@ -88,23 +88,19 @@ int reduce_static(lb_handle* h, unsigned char* base, double out[8]) {
   const double rho_mid = 0.5 * (h->d.rho_g + h->d.rho_l);
   k_reduce_partial<real, store_t><<<blocks, kReduceThreads, 0, h->stream>>>(
       f, rho, nx, ny, h->st, real(h->d.G2), rho_mid == rho_mid ? rho_mid : 1e300, partial);
-  k_reduce_final<<<1, 32, 0, h->stream>>>(partial, blocks, dout);
+  k_reduce_final<real><<<1, kFoldThreads, 0, h->stream>>>(partial, blocks, rho, size_t(ny / 2) * nx + nx / 2, dout);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return set_err(h, LB_ECUDA, "reduce kernels", e);
-  double res[kReduceSlots];
-  real probe[2];
-  e = cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&probe[0], rho + size_t(ny / 2) * nx + nx / 2, sizeof(real), cudaMemcpyDeviceToHost,
-                        h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&probe[1], rho, sizeof(real), cudaMemcpyDeviceToHost, h->stream);
+  double got[2 + kReduceSlots];
+  e = cudaMemcpyAsync(got, dout - 2, sizeof(got), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return set_err(h, LB_ECUDA, "reading the reduction", e);
+  const double *probe = got, *res = got + 2;
   out[0] = res[0];
   out[1] = res[1];
   out[2] = res[2];
-  out[3] = p_eos_host(h->cd, double(probe[0]));
-  out[4] = p_eos_host(h->cd, double(probe[1]));
+  out[3] = p_eos_host(h->cd, probe[0]);
+  out[4] = p_eos_host(h->cd, probe[1]);
   out[5] = res[3];
   out[6] = res[4];
   out[7] = res[5];
