@@ -44,14 +44,14 @@ KERNEL_SOURCES = ["paper_1809_02390_gb300/csrc/lbm_kernels.cuh", "paper_1809_023
 # layout and the hash of its sources (a changed kernel has no figure until recaptured).
 NCU_TRAFFIC = {
     # 2048^2 capture (profiles/k_step_tma_dyn_fp32_rows_2048_full.md) scaled x4 to 4096^2.
-    ("k_step_tma_dyn<f2>", "rows", "dbeb823cac5ca499"): 1020805120,
+    ("k_step_tma_dyn<f2>", "rows", "7004d44b0890cbfb"): 1019289600,
 }
 # The same for the D3Q19 step, keyed by the hash of its step code (csrc/lbm3d_step.cuh):
 # the 192^3 capture (profiles/k_d3_step_fp32_192cubed_full.md) scaled by the node
 # count to 256^3.
 KERNEL_SOURCES_D3Q19 = ["paper_1809_02390_gb300/csrc/lbm3d_step.cuh"]
 NCU_TRAFFIC_D3Q19 = {
-    ("k_d3_step<float, true>", "3c287283512da2cf"): 2676654080,
+    ("k_d3_step<float, true>", "79edb1409287a483"): 2664552978,
 }
 
 

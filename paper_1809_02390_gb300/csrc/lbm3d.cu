@@ -151,6 +151,7 @@ struct lb_d3_handle {
   int nz;
   void* f[2];
   int cur;
+  bool overlap;  // the steps' launches may overlap their predecessor's end (lbm_launch.cuh)
   cudaStream_t stream;
   CV3<r64> c64;
   CV3<f2> c32;
@@ -407,8 +408,8 @@ template <typename T, bool VEC>
 void launch_windows(lb_d3_handle* h, const CV3<typename ValOf<T>::V>& c) {
   const lb_params& p = h->p;
   const dim3 grid((p.nx + h->tw - 1) / h->tw, (p.ny + h->th - 1) / h->th, (h->nz + h->tz - 1) / h->tz);
-  k_d3_step<T, VEC><<<grid, Win3<T>::threads, Win3<T>::smem, h->stream>>>(
-      static_cast<const T*>(h->f[h->cur]), static_cast<T*>(h->f[1 - h->cur]), p.nx, p.ny, h->nz, h->tw,
+  lbm::launch_step_kernel(
+      h->overlap, k_d3_step<T, VEC>, grid, Win3<T>::threads, Win3<T>::smem, h->stream, static_cast<const T*>(h->f[h->cur]), static_cast<T*>(h->f[1 - h->cur]), p.nx, p.ny, h->nz, h->tw,
       h->th, h->tz, c, h->maps[h->cur], h->have_maps ? 1 : 0, h->wait_error);
 }
 
@@ -427,9 +428,9 @@ void launch_step(lb_d3_handle* h) {
     float* out = static_cast<float*>(h->f[1 - h->cur]);
     // 32-bit plane offsets while 19 nx ny nz < 2^31, 64-bit above.
     if (int64_t(Q) * p.nx * p.ny * h->nz >= (int64_t(1) << 31))
-      k_d3_pull<long long><<<grid, dim3(TX, kPullTY), 0, h->stream>>>(in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
+      lbm::launch_step_kernel(h->overlap, k_d3_pull<long long>, grid, dim3(TX, kPullTY), 0, h->stream, in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
     else
-      k_d3_pull<int><<<grid, dim3(TX, kPullTY), 0, h->stream>>>(in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
+      lbm::launch_step_kernel(h->overlap, k_d3_pull<int>, grid, dim3(TX, kPullTY), 0, h->stream, in, out, p.nx, p.ny, h->nz, h->tz, h->cpull);
   }
   h->cur = 1 - h->cur;
 }
@@ -603,6 +604,7 @@ int lb_d3_step(lb_d3_handle* h, int64_t nsteps) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;
   }
+  h->overlap = capture == cudaStreamCaptureStatusNone;
   while (capture == cudaStreamCaptureStatusNone && nsteps >= kD3GraphSteps && ensure_graph(h)) {
     const cudaError_t e = cudaGraphLaunch(h->exec[h->cur], h->stream);
     if (e != cudaSuccess) return fail3(h, LB_ECUDA, "step graph launch: %s", cudaGetErrorString(e));

@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(Win3<T>::threads, d3_blocks<T>())
   using W = Win3<T>;
   constexpr int L = Val<V>::lanes;
   constexpr bool kTensor = W::tensor && VEC;
+  lbm::follow_predecessor();
   extern __shared__ __align__(128) unsigned char dyn[];
   T* win = reinterpret_cast<T*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
   __shared__ T rho[3][W::ring_cells];
@@ -791,6 +792,7 @@ template <typename S>
 __global__ void __launch_bounds__(TX* kPullTY, 3)
     k_d3_pull(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int nz, int tz, C3<float> c) {
   using T = float;
+  lbm::follow_predecessor();
   __shared__ T pl[3][kPullHY][HX];
   const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * TX + tx;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * kPullTY, z0 = blockIdx.z * tz;

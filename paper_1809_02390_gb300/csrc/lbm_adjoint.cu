@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
     k_adj_fused(const store_t* __restrict__ s, const real* __restrict__ mu_in, const real* __restrict__ sb_in,
                 real* __restrict__ mu, real* __restrict__ sbar, double* __restrict__ partial, int accumulate, int nx,
                 int ny, VCoef<real> c) {
+  follow_predecessor();
   __shared__ real rs[kTileY + 2][kTileX + 2];   // density of s^n on tile + ring
   __shared__ real rb[kTileY + 2][kTileX + 2];   // rhob' on tile + ring
   __shared__ real sbx[kTileY + 4][kTileX + 4];  // Sb' on tile + two-node ring
@@ -396,6 +397,7 @@ __global__ void __launch_bounds__(kAdjThreads, 3)
               const __grid_constant__ CUtensorMap tsb, const float* __restrict__ s, const float* __restrict__ mu_in,
               const float* __restrict__ sb_in, float* __restrict__ mu, float* __restrict__ sbar,
               double* __restrict__ partial, int accumulate, int nx, int ny, VCoef<float> c, int* __restrict__ err) {
+  follow_predecessor();
   extern __shared__ __align__(128) unsigned char dyn[];
   float* const base = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
   const float* const muw = base + kAdjMuOff;
@@ -562,6 +564,7 @@ int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, dou
     }
   }
   k_adj_push<real><<<pgrd, blk, 0, h->stream>>>(static_cast<const real*>(lam), mu[0], sb[0], nx, ny);
+  const bool overlap = !stream_captured(h->stream);
   int cur = 0;
   for (int j = k - 1; j >= 0; --j) {
     bool done = false;
@@ -570,16 +573,16 @@ int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, dou
       if (staged && encode_population_map(&ts, const_cast<void*>(states[j]), nx, ny, nx, 4) &&
           encode_plane_map(&tm, mu[cur], nx, ny, 9, kMuCols, kMuRows) &&
           encode_plane_map(&tb, sb[cur], nx, ny, 2, kSbCols, kSbRows)) {
-        k_adj_tma<<<grd, kAdjThreads, kAdjStageSmem, h->stream>>>(
-            ts, tm, tb, static_cast<const float*>(states[j]), mu[cur], sb[cur], mu[1 - cur], sb[1 - cur], partial,
-            j < k - 1, nx, ny, *c, h->wait_error);
+        launch_step_kernel(overlap, k_adj_tma, grd, kAdjThreads, kAdjStageSmem, h->stream, ts, tm, tb,
+                           static_cast<const float*>(states[j]), mu[cur], sb[cur], mu[1 - cur], sb[1 - cur], partial,
+                           int(j < k - 1), nx, ny, *c, h->wait_error);
         done = true;
       }
     }
     if (!done)
-      k_adj_fused<real, store_t><<<grd, kAdjThreads, 0, h->stream>>>(
-          static_cast<const store_t*>(states[j]), mu[cur], sb[cur], mu[1 - cur], sb[1 - cur], partial, j < k - 1, nx,
-          ny, *c);
+      launch_step_kernel(overlap, k_adj_fused<real, store_t>, grd, kAdjThreads, 0, h->stream,
+                         static_cast<const store_t*>(states[j]), mu[cur], sb[cur], mu[1 - cur], sb[1 - cur], partial,
+                         int(j < k - 1), nx, ny, *c);
     cur = 1 - cur;
   }
   if (dtheta) k_adj_theta<<<1, 256, 0, h->stream>>>(partial, int(grd.x * grd.y), h->p.R_gas, dtheta);

@@ -95,6 +95,7 @@ __global__ void __launch_bounds__(TileShape<TY>::threads, MINB)
   static_assert(kCoefWords <= TileShape<TY>::threads, "one coefficient word per thread");
   __shared__ float rs[TY + 2][kTileX + 2];
   __shared__ LatCoef<f2> cs;
+  follow_predecessor();
   int t = blockIdx.x;
   if (t >= total_tiles) return;
   TileRec ti = tiles[t];
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(kFusedThreads, MINB)
                          const TileRec* __restrict__ tiles, const LatCoef<f2>* __restrict__ coef,
                          const CUtensorMap* __restrict__ maps, int total_tiles, VCoef<f2> common,
                          int* __restrict__ err, unsigned* __restrict__ queue, int rows) {
+  follow_predecessor();
   extern __shared__ __align__(128) unsigned char dyn[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
   __shared__ float rs[2][kTileY + 2][kTileX + 2];
@@ -352,13 +354,13 @@ __global__ void __launch_bounds__(kFusedThreads) k_batch_nonfinite(const float* 
 
 template <int TY, int MINB>
 void launch_shape(const float* in, float* out, const TileRec* tiles, const LatCoef<f2>* coef, int total, int bps,
-                  int sms, const VCoef<f2>& common, cudaStream_t st, int rows) {
+                  int sms, const VCoef<f2>& common, cudaStream_t st, int rows, bool overlap) {
   if (bps > 0)
-    k_step_batch<float, TY, MINB, true><<<bps * sms, TileShape<TY>::threads, 0, st>>>(in, out, tiles, coef, total,
-                                                                                        common, rows);
+    launch_step_kernel(overlap, k_step_batch<float, TY, MINB, true>, bps * sms, TileShape<TY>::threads, 0, st, in, out,
+                       tiles, coef, total, common, rows);
   else
-    k_step_batch<float, TY, MINB, false><<<total, TileShape<TY>::threads, 0, st>>>(in, out, tiles, coef, total,
-                                                                                     common, rows);
+    launch_step_kernel(overlap, k_step_batch<float, TY, MINB, false>, total, TileShape<TY>::threads, 0, st, in, out,
+                       tiles, coef, total, common, rows);
 }
 
 const void* batch_kernel(int shape) {
@@ -395,6 +397,7 @@ struct lb_batch {
   int rows;             // pools in the rows layout f[ny][9][sx] (else planes f[9][ny][sx])
   VCoef<f2> common;
   cudaStream_t stream;
+  bool overlap;  // launches may overlap their predecessor's end (lbm_launch.cuh)
   int sms;
   int shape;          // index into kShapeTY
   int blocks_per_sm;  // persistent grid = blocks_per_sm * sms
@@ -440,11 +443,11 @@ void launch_one(lb_batch* b, int from) {
     const int grid = std::min(b->blocks_per_sm * b->sms, total);
     const CUtensorMap* maps = b->d_maps + from * b->n;
     if (s == kShapeDyn)
-      k_step_batch_tma_dyn<3><<<grid, kFusedThreads, Win2<float>::smem, b->stream>>>(
-          in, out, tiles, b->d_coef, maps, total, b->common, b->d_err, b->d_queue, b->rows);
+      launch_step_kernel(b->overlap, k_step_batch_tma_dyn<3>, grid, kFusedThreads, Win2<float>::smem, b->stream, in, out,
+                         tiles, b->d_coef, maps, total, b->common, b->d_err, b->d_queue, b->rows);
     else if (s == kShapeDyn + 1)
-      k_step_batch_tma_dyn<2><<<grid, kFusedThreads, Win2<float>::smem, b->stream>>>(
-          in, out, tiles, b->d_coef, maps, total, b->common, b->d_err, b->d_queue, b->rows);
+      launch_step_kernel(b->overlap, k_step_batch_tma_dyn<2>, grid, kFusedThreads, Win2<float>::smem, b->stream, in, out,
+                         tiles, b->d_coef, maps, total, b->common, b->d_err, b->d_queue, b->rows);
     else if (s == kShapeTMA)
       k_step_batch_tma<3><<<grid, kFusedThreads, kTmaSmem, b->stream>>>(in, out, tiles, b->d_coef, maps, total,
                                                                          b->common, b->d_err, b->rows);
@@ -452,11 +455,14 @@ void launch_one(lb_batch* b, int from) {
       k_step_batch_tma<2><<<grid, kFusedThreads, kTmaSmem, b->stream>>>(in, out, tiles, b->d_coef, maps, total,
                                                                          b->common, b->d_err, b->rows);
   } else if (s == 0)
-    launch_shape<16, 4>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows);
+    launch_shape<16, 4>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
+                        b->overlap);
   else if (s == 1)
-    launch_shape<16, 3>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows);
+    launch_shape<16, 3>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
+                        b->overlap);
   else
-    launch_shape<32, 2>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows);
+    launch_shape<32, 2>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
+                        b->overlap);
 }
 
 int config_id(const lb_batch* b) { return b->shape * 64 + b->blocks_per_sm; }
@@ -754,6 +760,7 @@ int lb_batch_run(lb_batch* b, int64_t nsteps) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;
   }
+  b->overlap = capture == cudaStreamCaptureStatusNone;
   while (b->stream != nullptr && capture == cudaStreamCaptureStatusNone && nsteps >= kGraphSteps) {
     const int rc = ensure_graph(b, b->cur);
     if (rc != LB_OK) return rc;
@@ -778,6 +785,7 @@ int lb_batch_tune(lb_batch* b, int trial_steps, double* best_ms_per_step) {
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
     return berr(b, LB_ECUDA, "cudaEventCreate%s");
   float best = 1e30f;
+  b->overlap = true;
   int best_shape = b->shape, best_bps = b->blocks_per_sm;
   int64_t tuned_steps = 0;
   for (int s = 0; s < kShapes; ++s) {

@@ -212,8 +212,8 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
     const dim3 grd((nx + kTileX - 1) / kTileX, (ny + TY - 1) / TY);
     if constexpr (sizeof(store_t) <= 4 && std::is_same<V, f2>::value) {
       if (h->use_tma && h->use_dyn) {
-        k_step_tma_dyn<V, store_t><<<h->dyn_grid, kFusedThreads, Win2<store_t>::smem, h->stream>>>(
-            h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd, h->queue);
+        launch_step_kernel(
+            h->overlap, k_step_tma_dyn<V, store_t>, h->dyn_grid, kFusedThreads, Win2<store_t>::smem, h->stream, h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd, h->queue);
         return;
       }
       if (h->use_tma) {
@@ -222,7 +222,8 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
         return;
       }
     }
-    k_step_fused<V, store_t><<<grd, TileShape<TY>::threads, 0, h->stream>>>(fin, fout, nx, ny, h->st, cv, rnd);
+    launch_step_kernel(h->overlap, k_step_fused<V, store_t, TY>, grd, TileShape<TY>::threads, 0, h->stream, fin, fout, nx, ny,
+                       h->st, cv, rnd);
   } else {
     real* rho = static_cast<real*>(h->scratch);
     const dim3 blk(32, 8), grd((nx + 31) / 32, (ny + 7) / 8);
@@ -772,6 +773,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
   }
+  h->overlap = capture == cudaStreamCaptureStatusNone;
   if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= kResMinSteps && capture == cudaStreamCaptureStatusNone) {
     LB_CUDA(h, res_run(h, nsteps, nullptr, 1));
     return LB_OK;
@@ -818,6 +820,7 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
     cudaGetLastError();
     capture = cudaStreamCaptureStatusActive;
   }
+  h->overlap = capture == cudaStreamCaptureStatusNone;
   if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= 2 && capture == cudaStreamCaptureStatusNone) {
     LB_CUDA(h, res_run(h, nsteps, states, every));
     return LB_OK;

@@ -56,6 +56,7 @@ struct lb_handle {
   void* res_mail;         // exchange words (end of the scratch buffer)
   unsigned res_epoch;     // numbers up to this one have been used
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
+  bool overlap;           // the steps' launches may overlap their predecessor's end (lbm_launch.cuh)
   int graph_k;            // while capturing: the place of the launch in the graph (else -1)
   lbm::VCoef<float> cf;  // FP32 scalar (two-pass variant, moments)
   lbm::VCoef<lbm::f2> c2;     // FP32 pairs (fused variant)

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm_device.cuh"
+#include "lbm_launch.cuh"
 
 namespace lbm {
 
@@ -300,6 +301,7 @@ template <typename V, typename store_t, int TY = fused_rows<V>()>
 __global__ void __launch_bounds__(TileShape<TY>::threads, fused_min_blocks<V>() * (kTileY / TY))
     k_step_fused(const store_t* __restrict__ fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
                  VCoef<V> c, Rounding rnd) {
+  follow_predecessor();
   rnd = resolve(rnd);
   __shared__ __align__(16) typename LaneType<V>::type rs[TY + 2][kTileX + 2];
   constexpr bool XP = xpairs<store_t>() && Lanes<V>::n == 2;
