@@ -44,7 +44,7 @@ KERNEL_SOURCES = ["paper_1809_02390_gb300/csrc/lbm_kernels.cuh", "paper_1809_023
 # layout and the hash of its sources (a changed kernel has no figure until recaptured).
 NCU_TRAFFIC = {
     # 2048^2 capture (profiles/k_step_tma_dyn_fp32_rows_2048_full.md) scaled x4 to 4096^2.
-    ("k_step_tma_dyn<f2>", "rows", "7004d44b0890cbfb"): 1019289600,
+    ("k_step_tma_dyn<f2>", "rows", "dca95e80b9112257"): 1020884992,
 }
 # The same for the D3Q19 step, keyed by the hash of its step code (csrc/lbm3d_step.cuh):
 # the 192^3 capture (profiles/k_d3_step_fp32_192cubed_full.md) scaled by the node
@@ -590,7 +590,9 @@ def run_ours(args):
     lat = Lattice(rho0, precision=main_prec, variant=main_var, Tr=TR, layout=args.layout)
     if args.dispatch == "static" and capi.lb_tile_dispatch(lat.h):
         capi.lb_set_tile_dispatch(lat.h, False)
-    kernel = ("k_step_tma_dyn<f2>" if capi.lb_tile_dispatch(lat.h) else "k_step_tma<f2>") if capi.lb_uses_tma(lat.h) \
+    tensor = capi.lb_uses_tma(lat.h) and (args.dispatch == "static" or
+                                          2 * lat.f_a.numel() * lat.f_a.element_size() > 100 << 20)
+    kernel = ("k_step_tma_dyn<f2>" if capi.lb_tile_dispatch(lat.h) else "k_step_tma<f2>") if tensor \
         else ("k_step_fused<f2,float>" if main_var == "fused" else "k_density + k_collide_rho")
     lat.step(args.warmup)
     barrier(world)

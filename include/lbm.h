@@ -158,9 +158,9 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
             size_t scratch_bytes, const double* rho0, int rho0_on_device, void* stream);
 
 /* Advances nsteps >= 0 time steps (Eq. 13 + supplement Eq. 2) on the stream.
- * Asynchronous.  A fused lattice whose populations fit the SMs' shared memory twice
- * (FP64 to about 485^2, FP32 610^2, FP16 860^2) takes calls of at least four steps in
- * one cooperative launch that keeps it there (same bits; waits between its blocks are
+ * Asynchronous.  A small fused lattice (FP64 to about 485^2, FP32 and FP16 to 340,000
+ * nodes) takes calls of several steps (at least 4, FP32 and FP16 12) in one cooperative
+ * launch that keeps it in the SMs' shared memory (same bits; waits between its blocks are
  * bounded at 10 s and reported by lb_status), unless lb_set_step_blocks or
  * lb_set_tile_dispatch ask for another form.  Else runs of 64 steps replay a CUDA graph that the handle captures on
  * first use (again after lb_set_step_blocks or lb_set_tile_dispatch change the
@@ -366,7 +366,9 @@ int lb_wait_selftest(lb_handle* h, long long polls);
 
 /* 1 if the handle's fused step stages populations with tensor copies (TMA):
  * FP32 storage with nx a multiple of 4 and nx >= 104, or FP16 storage with nx a
- * multiple of 8 and nx >= 112; ny >= 50.  Else 0. */
+ * multiple of 8 and nx >= 112; ny >= 50.  Else 0.  (A lattice whose two buffers are at most
+ * 100 MB steps by plain loads all the same, which L2 serves faster, unless
+ * lb_set_step_blocks or lb_set_tile_dispatch was called.  Same bits.) */
 int lb_uses_tma(const lb_handle* h);
 
 /* How the tensor-copy step hands tiles to its persistent blocks.  1 (the default

@@ -195,6 +195,12 @@ constexpr size_t kQueueBytes = 256;  // tile tickets of the dynamic tensor-copy 
 // steps are then launched one by one).
 size_t base_scratch_bytes(const lb_params* p) { return rho_plane_bytes(p) + reduce_bytes() + kQueueBytes; }
 
+// Whether steps take the tensor-copy kernel: h->use_tma, unless the lattice is small
+// enough for the plain one and no launch form was asked for.
+bool tensor_step(const lb_handle* h) {
+  return h->use_tma && (!h->plain_small || h->forced_blocks || h->forced_dispatch);
+}
+
 template <typename V, typename real, typename store_t>
 void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
   const store_t* fin = static_cast<const store_t*>(h->f[h->cur]);
@@ -208,22 +214,21 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
     rnd.k = h->graph_k;
   }
   if (h->variant == LB_FUSED) {
-    constexpr int TY = fused_rows<V>();
-    const dim3 grd((nx + kTileX - 1) / kTileX, (ny + TY - 1) / TY);
+    const dim3 grd((nx + kTileX - 1) / kTileX, (ny + kFusedRows - 1) / kFusedRows);
     if constexpr (sizeof(store_t) <= 4 && std::is_same<V, f2>::value) {
-      if (h->use_tma && h->use_dyn) {
-        launch_step_kernel(
-            h->overlap, k_step_tma_dyn<V, store_t>, h->dyn_grid, kFusedThreads, Win2<store_t>::smem, h->stream, h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd, h->queue);
+      if (tensor_step(h) && h->use_dyn) {
+        launch_step_kernel(h->overlap, k_step_tma_dyn<V, store_t>, h->dyn_grid, kFusedThreads, Win2<store_t>::smem,
+                           h->stream, h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd, h->queue);
         return;
       }
-      if (h->use_tma) {
+      if (tensor_step(h)) {
         k_step_tma<V, store_t, false><<<h->tma_grid, kFusedThreads, Win<store_t>::smem, h->stream>>>(
             h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd);
         return;
       }
     }
-    launch_step_kernel(h->overlap, k_step_fused<V, store_t, TY>, grd, TileShape<TY>::threads, 0, h->stream, fin, fout, nx, ny,
-                       h->st, cv, rnd);
+    launch_step_kernel(h->overlap, k_step_fused<V, store_t>, grd, TileShape<kFusedRows>::threads, 0, h->stream, fin,
+                       fout, nx, ny, h->st, cv, rnd);
   } else {
     real* rho = static_cast<real*>(h->scratch);
     const dim3 blk(32, 8), grd((nx + 31) / 32, (ny + 7) / 8);
@@ -480,6 +485,12 @@ int configure(lb_handle* h) {
     if (h->tma_grid_auto > tiles) h->tma_grid_auto = tiles;
     h->tma_grid = h->tma_grid_auto;
   }
+  // Lattices whose two buffers stay in L2 (129 MB) run k_step_fused all the same: its many
+  // small blocks hide L2's latency better than two staged tiles a block.  us a step, plain
+  // against tensor copies: FP32 512^2 4.7 / 6.7, 1024^2 13.6 / 16.2, 1200 x 1104 (95 MB) 19.1 /
+  // 19.7, 1304 x 1200 (113 MB) 23.3 / 23.0, 2048^2 59.5 / 50.9; FP16 1024^2 14.7 / 17.1, 1600^2
+  // (92 MB) 34.5 / 34.3, 2048 x 1400 (103 MB) 38.4 / 37.8.
+  h->plain_small = size_t(2) * lb_state_bytes(&h->p) <= (size_t(100) << 20);
   // Dynamic tile dispatch: needs the ticket words at the end of the scratch buffer.
   h->use_dyn = false;
   h->queue = h->scratch ? reinterpret_cast<unsigned*>(static_cast<char*>(h->scratch) + rho_plane_bytes(&h->p) +
@@ -696,8 +707,12 @@ namespace {
 
 // Steps per captured graph (even, so a replay ends on the buffer it started from).
 constexpr int kStepGraph = 64;
-// Fewest steps of a call that run resident.
-constexpr int64_t kResMinSteps = 4;
+// Fewest steps of a call that run resident: the launch costs some 8 us more than an
+// ordinary one (load, store, cooperative start), a step less (FP32 256^2 2.15 against 2.74 us,
+// 400^2 3.0 / 4.2, FP16 256^2 2.5 / 3.35: from 12 or 13, 8 and 8 steps; FP64 64^2 7.6 / 21.5).
+int64_t res_min_steps(const lb_handle* h) { return h->p.precision == LB_FP64 ? 4 : 12; }
+// The same for runs that record states.
+int64_t res_min_record(const lb_handle* h) { return h->p.precision == LB_FP64 ? 2 : 12; }
 
 void launch_one_step(lb_handle* h) {
   switch (h->p.precision) {
@@ -709,7 +724,7 @@ void launch_one_step(lb_handle* h) {
 
 // The launch configuration a graph bakes in: kernel form and grid sizes.
 long long step_config(const lb_handle* h) {
-  return (long long)h->variant | ((long long)h->use_tma << 2) | ((long long)h->use_dyn << 3) |
+  return (long long)h->variant | ((long long)tensor_step(h) << 2) | ((long long)h->use_dyn << 3) |
          ((long long)h->tma_grid << 4) | ((long long)h->dyn_grid << 34);
 }
 
@@ -774,7 +789,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= kResMinSteps && capture == cudaStreamCaptureStatusNone) {
+  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_steps(h) && capture == cudaStreamCaptureStatusNone) {
     LB_CUDA(h, res_run(h, nsteps, nullptr, 1));
     return LB_OK;
   }
@@ -821,7 +836,7 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
     capture = cudaStreamCaptureStatusActive;
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= 2 && capture == cudaStreamCaptureStatusNone) {
+  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_record(h) && capture == cudaStreamCaptureStatusNone) {
     LB_CUDA(h, res_run(h, nsteps, states, every));
     return LB_OK;
   }
@@ -1017,6 +1032,7 @@ int lb_set_tile_dispatch(lb_handle* h, int dynamic) {
     return fail(h, LB_ENOTSUP, "dynamic dispatch needs the tensor-copy step and the scratch buffer");
   h->use_dyn = dynamic != 0;
   h->forced_walk = h->use_tma && !dynamic;
+  h->forced_dispatch = true;
   return LB_OK;
 }
 

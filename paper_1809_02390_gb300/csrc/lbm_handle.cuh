@@ -51,6 +51,8 @@ struct lb_handle {
   // Resident run (lbm_resident.cu): many steps per launch on lattices that fit the SMs'
   // shared memory.
   bool use_res;
+  bool plain_small;       // small enough for k_step_fused although tensor copies could serve it
+  bool forced_dispatch;   // lb_set_tile_dispatch was called
   bool forced_blocks, forced_walk;  // lb_set_step_blocks, lb_set_tile_dispatch fixed another launch form
   lbm::ResPlan res;
   void* res_mail;         // exchange words (end of the scratch buffer)

@@ -71,17 +71,6 @@ __device__ __forceinline__ double sum9(const double (&f)[9]) {
 // is one read and one write of every population; the ring re-reads hit L2.
 constexpr int kTileX = 32, kTileY = 16, kTileRows = 2;
 constexpr int kRowStride = kTileY / kTileRows;  // 8
-#ifndef LBM_FUSED_MIN_BLOCKS
-#define LBM_FUSED_MIN_BLOCKS 4
-#endif
-// Resident blocks per SM the register budget must allow: 4 for the FP32-pair
-// kernels (64 registers; the kernel is latency-bound, so the extra resident warps
-// outweigh a few spilled registers), 2 for FP64.
-template <typename V>
-constexpr int fused_min_blocks() {
-  return sizeof(typename LaneType<V>::type) == 8 ? 2 : LBM_FUSED_MIN_BLOCKS;
-}
-
 template <int TY>
 struct TileShape {
   static constexpr int threads = kTileX * TY / kTileRows;
@@ -289,24 +278,32 @@ __device__ __forceinline__ void step_tile(const store_t* __restrict__ fin, store
   collide_tile<V, store_t, TY, XP>(f, fout, nx, ny, st, c, l, x0, y0, rs, rnd);
 }
 
-// TY: rows of a tile.  FP64 steps take 8 (fused_rows): the FP64 pipe bounds them, so an
-// SM's time is its number of tiles, and half-size tiles spread more evenly (1024^2 on
-// 152 SMs: at most 27 of 26.9 tiles on average, against 14 of 13.5) at the price of one
-// more density addition per node.
-template <typename V>
-constexpr int fused_rows() {
-  return sizeof(typename LaneType<V>::type) == 8 ? 8 : kTileY;
+// Rows of a tile of k_step_fused.  FP64: its pipe is the bound, so an SM's time is its
+// number of tiles, and half-size tiles spread more evenly (1024^2 on 152 SMs: at most 27 of
+// 26.9 tiles on average, against 14 of 13.5) at the price of one more density addition per
+// node.  FP32 and FP16: more, smaller blocks fill each other's load phases and the last
+// wave (FP32 1003 x 517 8.8 -> 7.9 us a step, 4095^2 261 -> 227, both at 80 registers).
+constexpr int kFusedRows = 8;
+// Resident blocks per SM the register budget must allow.  FP32: 6 (80 registers).  With 64
+// registers the collision spills 124 bytes a thread, whose stores went through to L2 (twice
+// the write traffic of the step itself) and bounded it: 1003 x 517 10.5 us a step against
+// 7.9, 4095^2 290 against 227; 7 (72 registers, 68 bytes) 8.6 and 242.  FP16 spills less and
+// has more conversions to hide: 7 blocks, 4095^2 238 us (6: 258, 8: 263), 1003 x 517 9.8
+// (10.0, 9.1).
+template <typename V, typename store_t>
+constexpr int fused_min_blocks() {
+  return sizeof(typename LaneType<V>::type) == 8 ? 4 : sizeof(store_t) == 2 ? 7 : 6;
 }
-template <typename V, typename store_t, int TY = fused_rows<V>()>
-__global__ void __launch_bounds__(TileShape<TY>::threads, fused_min_blocks<V>() * (kTileY / TY))
+template <typename V, typename store_t>
+__global__ void __launch_bounds__(TileShape<kFusedRows>::threads, fused_min_blocks<V, store_t>())
     k_step_fused(const store_t* __restrict__ fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
                  VCoef<V> c, Rounding rnd) {
   follow_predecessor();
   rnd = resolve(rnd);
-  __shared__ __align__(16) typename LaneType<V>::type rs[TY + 2][kTileX + 2];
+  __shared__ __align__(16) typename LaneType<V>::type rs[kFusedRows + 2][kTileX + 2];
   constexpr bool XP = xpairs<store_t>() && Lanes<V>::n == 2;
-  step_tile<V, store_t, TY, NoHook, XP>(fin, fout, nx, ny, st, c, lattice_part(c), blockIdx.x * kTileX,
-                                        blockIdx.y * TY, rs, NoHook(), rnd);
+  step_tile<V, store_t, kFusedRows, NoHook, XP>(fin, fout, nx, ny, st, c, lattice_part(c), blockIdx.x * kTileX,
+                                        blockIdx.y * kFusedRows, rs, NoHook(), rnd);
 }
 
 // Two-pass variant, pass 1: density plane rho_dev(x) = sum_i fbar_i(x - e_i).
