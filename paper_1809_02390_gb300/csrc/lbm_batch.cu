@@ -96,9 +96,15 @@ __global__ void __launch_bounds__(TileShape<TY>::threads, MINB)
   __shared__ float rs[TY + 2][kTileX + 2];
   __shared__ LatCoef<f2> cs;
   follow_predecessor();
-  int t = blockIdx.x;
+  constexpr bool kHalves = TY < kTileY;  // two blocks share a record of 16 rows
+  static_assert(!kHalves || (TY * 2 == kTileY && !PERSIST), "halves of 16-row tiles, a block each");
+  int t = kHalves ? blockIdx.x >> 1 : blockIdx.x;
   if (t >= total_tiles) return;
   TileRec ti = tiles[t];
+  if constexpr (kHalves) {
+    ti.y0 += (blockIdx.x & 1) * TY;
+    if (ti.y0 >= ti.ny) return;
+  }
   int word = threadIdx.x < kCoefWords ? reinterpret_cast<const int*>(coef + ti.lat)[threadIdx.x] : 0;
   if constexpr (!PERSIST) {  // one block per tile
     step_tile<f2, store_t, TY>(pool_in + ti.offset, pool_out + ti.offset, ti.nx, ti.ny,
@@ -457,6 +463,11 @@ void launch_one(lb_batch* b, int from) {
   } else if (s == 0)
     launch_shape<16, 4>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
                         b->overlap);
+  else if (s == 1 && b->blocks_per_sm == 0)
+    // One block per half tile: 8 rows, 6 blocks per SM at 80 registers.  Smaller blocks hide
+    // each other's loads (48 lattices, 0.92 M nodes: 16.9 -> 14.4 us a step).
+    launch_step_kernel(b->overlap, k_step_batch<float, 8, 6, false>, 2 * total, TileShape<8>::threads, 0, b->stream, in,
+                       out, tiles, b->d_coef, total, b->common, b->rows);
   else if (s == 1)
     launch_shape<16, 3>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
                         b->overlap);
@@ -732,11 +743,11 @@ int lb_batch_init(lb_batch** out, const lb_params* ps, int n, void* pool_a, void
     return bail(LB_ECUDA, msg);
   }
   // Launch form until lb_batch_tune or lb_batch_set_config choose one (the results are the
-  // same).  Pools that L2 holds: one block per tile at 80 registers (48 lattices, 0.92 M
-  // nodes: 16.9 us a step, tickets 20.8, the persistent plain-load grid 21.6); larger
-  // ones: tensor copies with tiles by ticket (6.7 M nodes: 96.9 us, one block per tile
-  // 111, the plain-load grid 139).  The line lies at 100 MB of the 129 MB of L2: 1.18 M
-  // nodes (85 MB) 21.5 against 23.7 us, 4.9 M (351 MB) 81.5 against 72.2.
+  // same).  Pools that L2 holds: one block per half tile at 80 registers (us a step, against
+  // tickets and the persistent plain-load grid: 0.92 M nodes 14.4, 20.3, 24.8; 1.18 M 19.5,
+  // 23.3, 27.6); larger ones: tensor copies with tiles by ticket (4.9 M nodes 71.7, half
+  // tiles 73.7, the grid 101.7; 6.7 M 96.2, 101.1, 138.9).  The line lies at 100 MB of the
+  // 129 MB of L2 (1.46 M nodes), where one lattice's step changes sides.
   b->shape = 1;
   b->blocks_per_sm = 0;
   if (b->tma_ok && 2 * off * sizeof(float) > (size_t(100) << 20)) {

@@ -54,3 +54,21 @@ def test_equals_the_tensor_copy_step(precision, nx, ny, layout):
     capi.lb_status(b.h)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("layout", ["planes", "rows"])
+def test_half_tiles_of_a_batch(layout):
+    """One block per tile in the 80-register form takes 8-row halves of the 16-row tiles:
+    lattices whose last tile is a half, part of one or whole."""
+    from paper_1809_02390_gb300 import Batch, Lattice
+
+    sizes = [(33, 8), (40, 9), (64, 16), (31, 17), (65, 24), (130, 31)]
+    b = Batch([_rho(*s) for s in sizes], [dict(Tr=0.8, layout=layout) for _ in sizes])
+    b.set_config(1, 0)
+    b.run(64 + 3)
+    for i, s in enumerate(sizes):
+        lat = Lattice(_rho(*s), precision="fp32", Tr=0.8)
+        lat.step(64 + 3)
+        assert torch.equal(b.state(i), lat.state()), s
+        lat.close()
+    b.close()
