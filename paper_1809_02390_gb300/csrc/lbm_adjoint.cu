@@ -181,33 +181,41 @@ __global__ void k_adj_theta(const double* __restrict__ partial, int nblocks, dou
 // k_adj_local + k_adj_transpose.  The VJP runs node by node in scalar FP32: as a
 // packed pair (two nodes per FFMA2) its live set needs 128 registers (2 blocks/SM)
 // or spills 350 bytes per thread at 80, and either way the step was 20% slower.
-// Resident blocks per SM: 3 for FP32 (<= 85 registers), 1 for FP64.
-template <typename real>
+// TY rows a tile, ROWS nodes a thread.  FP64 takes (16, 2).  FP32, per step:
+//   (8, 1), two blocks per SM, while every tile is resident at once: a block is a chain of
+//     latencies and one node halves its longest part (64^2 5.0 -> 3.7 us, 256^2 5.2 -> 4.6;
+//     with three waves of blocks its extra barriers cost more, 400^2 9.3 -> 10.9);
+//   (8, 2), six blocks per SM, above: 301^2 7.0 -> 6.0 us, 512^2 12.4 -> 12.1, 400^2 9.3 both;
+//   (16, 2), three, with a scratch that has room only for the partials of 16-row tiles.
+template <int TY, int ROWS>
+constexpr int adj_threads = kTileX * TY / ROWS;
+template <typename real, int TY, int ROWS>
 constexpr int adj_min_blocks() {
-  return sizeof(real) == 8 ? 1 : 3;
+  return sizeof(real) == 8 ? 1 : TY == 16 ? 3 : ROWS == 1 ? 2 : 6;
 }
 
-template <typename real, typename store_t>
-__global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
+template <typename real, typename store_t, int TY, int ROWS>
+__global__ void __launch_bounds__(adj_threads<TY, ROWS>, adj_min_blocks<real, TY, ROWS>())
     k_adj_fused(const store_t* __restrict__ s, const real* __restrict__ mu_in, const real* __restrict__ sb_in,
                 real* __restrict__ mu, real* __restrict__ sbar, double* __restrict__ partial, int accumulate, int nx,
                 int ny, VCoef<real> c) {
+  constexpr int NT = adj_threads<TY, ROWS>;
   follow_predecessor();
-  __shared__ real rs[kTileY + 2][kTileX + 2];   // density of s^n on tile + ring
-  __shared__ real rb[kTileY + 2][kTileX + 2];   // rhob' on tile + ring
-  __shared__ real sbx[kTileY + 4][kTileX + 4];  // Sb' on tile + two-node ring
-  __shared__ real sby[kTileY + 4][kTileX + 4];
+  __shared__ real rs[TY + 2][kTileX + 2];   // density of s^n on tile + ring
+  __shared__ real rb[TY + 2][kTileX + 2];   // rhob' on tile + ring
+  __shared__ real sbx[TY + 4][kTileX + 4];  // Sb' on tile + two-node ring
+  __shared__ real sby[TY + 4][kTileX + 4];
   // mu'_i(x + e_i) at the tile's nodes, staged for FP32 (in FP64 the 37 KB would
   // exceed the static shared-memory limit next to the rest; FP64 reads directly).
   constexpr bool kStageMu = sizeof(real) == 4;
-  __shared__ real mus[kStageMu ? 9 : 1][kTileY][kTileX];
-  __shared__ real red[kAdjThreads / 32][3];
+  __shared__ real mus[kStageMu ? 9 : 1][TY][kTileX];
+  __shared__ real red[NT / 32][3];
   const int tx = threadIdx.x & (kTileX - 1), ty = threadIdx.x / kTileX;
-  const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * kTileY;
+  const int x0 = blockIdx.x * kTileX, y0 = blockIdx.y * TY;
   const int plane = nx * ny;
   // Every coordinate below lies in [-2, n + 33); one conditional wrap suffices
   // unless the lattice is smaller than a tile plus its two-node ring.
-  const bool small = nx < kTileX + 4 || ny < kTileY + 4;
+  const bool small = nx < kTileX + 4 || ny < TY + 4;
   auto wr = [&](int v, int n) { return small ? wrap(v, n) : wrap1(v, n); };
   const int gx = x0 + tx;
   const int xc = wr(gx, nx);
@@ -217,8 +225,8 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
   // nodes (wrapped coordinates also past a ragged edge: in bounds, unused), and Sb'
   // on the tile with its two-node ring.
 #pragma unroll
-  for (int k = 0; k < (kStageMu ? kTileRows : 0); ++k) {
-    const int ly = ty + k * kRowStride;
+  for (int k = 0; k < (kStageMu ? ROWS : 0); ++k) {
+    const int ly = ty + k * (TY / ROWS);
     const int yc = wr(y0 + ly, ny);
     const int ym = yc == 0 ? ny - 1 : yc - 1, yp = yc == ny - 1 ? 0 : yc + 1;
     const int oc = yc * nx, om = ym * nx, op = yp * nx;
@@ -232,31 +240,31 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
     cp_async_elem(&mus[7][ly][tx], mu_in + (7 * plane + om + xm));
     cp_async_elem(&mus[8][ly][tx], mu_in + (8 * plane + om + xp));
   }
-  for (int t = threadIdx.x; t < (kTileY + 4) * (kTileX + 4); t += kAdjThreads) {
+  for (int t = threadIdx.x; t < (TY + 4) * (kTileX + 4); t += NT) {
     const int wy = t / (kTileX + 4), wx = t - wy * (kTileX + 4);
     const int o = wr(y0 - 2 + wy, ny) * nx + wr(x0 - 2 + wx, nx);
     cp_async_elem(&sbx[wy][wx], sb_in + o);
     cp_async_elem(&sby[wy][wx], sb_in + (plane + o));
   }
   cp_async_commit();
-  real f[kTileRows][9];
+  real f[ROWS][9];
 #pragma unroll
-  for (int k = 0; k < kTileRows; ++k) {
-    const int gy = y0 + ty + k * kRowStride;
+  for (int k = 0; k < ROWS; ++k) {
+    const int gy = y0 + ty + k * (TY / ROWS);
     pull_row(s, plane, nx, ny, wr(gy, ny), xm, xc, xp, f[k]);
   }
 #pragma unroll
-  for (int k = 0; k < kTileRows; ++k) rs[ty + k * kRowStride + 1][tx + 1] = sum9(f[k]);
-  for (int t = threadIdx.x; t < 2 * (kTileX + 2) + 2 * kTileY; t += kAdjThreads) {
+  for (int k = 0; k < ROWS; ++k) rs[ty + k * (TY / ROWS) + 1][tx + 1] = sum9(f[k]);
+  for (int t = threadIdx.x; t < 2 * (kTileX + 2) + 2 * TY; t += NT) {
     int wx, wy;
     if (t < kTileX + 2) {
       wx = t, wy = 0;
     } else if (t < 2 * (kTileX + 2)) {
-      wx = t - (kTileX + 2), wy = kTileY + 1;
-    } else if (t < 2 * (kTileX + 2) + kTileY) {
+      wx = t - (kTileX + 2), wy = TY + 1;
+    } else if (t < 2 * (kTileX + 2) + TY) {
       wx = 0, wy = t - 2 * (kTileX + 2) + 1;
     } else {
-      wx = kTileX + 1, wy = t - 2 * (kTileX + 2) - kTileY + 1;
+      wx = kTileX + 1, wy = t - 2 * (kTileX + 2) - TY + 1;
     }
     const int hx = wr(x0 - 1 + wx, nx), hy = wr(y0 - 1 + wy, ny);
     real g[9];
@@ -267,7 +275,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
   __syncthreads();
   // rhob'(y) = sum_j omega_j e_j . Sb'(y - e_j) on tile + ring (smem index of y is (wy + 1, wx + 1)).
   const real third = real(1.0 / 3.0), twelfth = real(1.0 / 12.0);
-  for (int t = threadIdx.x; t < (kTileY + 2) * (kTileX + 2); t += kAdjThreads) {
+  for (int t = threadIdx.x; t < (TY + 2) * (kTileX + 2); t += NT) {
     const int wy = t / (kTileX + 2), wx = t - wy * (kTileX + 2);
     const int cy = wy + 1, cx = wx + 1;
     const real ax = sbx[cy][cx - 1] - sbx[cy][cx + 1];
@@ -283,8 +291,8 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
   // is slow on this GPU); warp partials are folded in FP64.
   real acc[3] = {real(0), real(0), real(0)};
 #pragma unroll
-  for (int k = 0; k < kTileRows; ++k) {
-    const int ly = ty + k * kRowStride + 1, lx = tx + 1;
+  for (int k = 0; k < ROWS; ++k) {
+    const int ly = ty + k * (TY / ROWS) + 1, lx = tx + 1;
     const int gy = y0 + ly - 1;
     if (gx >= nx || gy >= ny) continue;
     real Sx, Sy;
@@ -342,7 +350,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_min_blocks<real>())
     // The block's partial in the compute type, widened once: one FP64 add per
     // block and parameter per step.
     real v = real(0);
-    for (int j = 0; j < kAdjThreads / 32; ++j) v += red[j][threadIdx.x];
+    for (int j = 0; j < NT / 32; ++j) v += red[j][threadIdx.x];
     // Each block owns its slot; successive steps on one stream accumulate in order.
     double* slot = partial + (size_t(blockIdx.y) * gridDim.x + blockIdx.x) * 3 + threadIdx.x;
     *slot = accumulate ? *slot + double(v) : double(v);
@@ -519,15 +527,16 @@ size_t adj_scratch_bytes(const lb_params* p, size_t real_bytes) {
   return ((11 * N * real_bytes + 255) / 256) * 256 + blocks * 3 * sizeof(double);
 }
 
-// Two (mu, Sb) sets (ping-pong) + per-block partials.
-size_t adj_steps_scratch_bytes(const lb_params* p, size_t real_bytes) {
+// Two (mu, Sb) sets (ping-pong) + partials of blocks of `rows` lattice rows.
+size_t adj_steps_scratch_bytes(const lb_params* p, size_t real_bytes, int rows) {
   const size_t N = size_t(p->nx) * p->ny;
-  const size_t blocks = size_t((p->nx + kTileX - 1) / kTileX) * ((p->ny + kTileY - 1) / kTileY);
+  const size_t blocks = size_t((p->nx + kTileX - 1) / kTileX) * ((p->ny + rows - 1) / rows);
   return 2 * ((11 * N * real_bytes + 255) / 256) * 256 + blocks * 3 * sizeof(double);
 }
 
 template <typename real, typename store_t>
-int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, double* dtheta, void* scratch) {
+int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, double* dtheta, void* scratch,
+                  size_t scratch_bytes) {
   const int nx = h->p.nx, ny = h->p.ny;
   const size_t N = size_t(nx) * ny;
   const size_t set = ((11 * N * sizeof(real) + 255) / 256) * 256;
@@ -563,6 +572,9 @@ int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, dou
       staged = true;
     }
   }
+  // Else k_adj_fused with 8-row tiles where the scratch holds their partials.
+  const bool halves = sizeof(real) == 4 && !staged && scratch_bytes >= adj_steps_scratch_bytes(&h->p, sizeof(real), 8);
+  const dim3 hgrd(grd.x, (ny + 7) / 8);
   k_adj_push<real><<<pgrd, blk, 0, h->stream>>>(static_cast<const real*>(lam), mu[0], sb[0], nx, ny);
   const bool overlap = !stream_captured(h->stream);
   int cur = 0;
@@ -579,13 +591,24 @@ int adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, dou
         done = true;
       }
     }
-    if (!done)
-      launch_step_kernel(overlap, k_adj_fused<real, store_t>, grd, kAdjThreads, 0, h->stream,
-                         static_cast<const store_t*>(states[j]), mu[cur], sb[cur], mu[1 - cur], sb[1 - cur], partial,
-                         int(j < k - 1), nx, ny, *c);
+    auto fused = [&](auto kernel, dim3 grid, int threads) {
+      launch_step_kernel(overlap, kernel, grid, threads, 0, h->stream, static_cast<const store_t*>(states[j]), mu[cur],
+                         sb[cur], mu[1 - cur], sb[1 - cur], partial, int(j < k - 1), nx, ny, *c);
+    };
+    if constexpr (sizeof(real) == 4) {
+      if (halves) {
+        if (size_t(hgrd.x) * hgrd.y <= size_t(2) * sms)
+          fused(k_adj_fused<real, store_t, 8, 1>, hgrd, adj_threads<8, 1>);
+        else
+          fused(k_adj_fused<real, store_t, 8, 2>, hgrd, adj_threads<8, 2>);
+        done = true;
+      }
+    }
+    if (!done) fused(k_adj_fused<real, store_t, kTileY, kTileRows>, grd, kAdjThreads);
     cur = 1 - cur;
   }
-  if (dtheta) k_adj_theta<<<1, 256, 0, h->stream>>>(partial, int(grd.x * grd.y), h->p.R_gas, dtheta);
+  if (dtheta)
+    k_adj_theta<<<1, 256, 0, h->stream>>>(partial, int(halves ? hgrd.x * hgrd.y : grd.x * grd.y), h->p.R_gas, dtheta);
   k_adj_transpose<real><<<grd, kAdjThreads, 0, h->stream>>>(mu[cur], sb[cur], static_cast<real*>(lam), nx, ny);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
@@ -657,7 +680,7 @@ int lb_adjoint_step(lb_handle* h, const void* f_state, const void* lam_in, void*
 
 size_t lb_adjoint_steps_scratch_bytes(const lb_params* p) {
   if (!p || p->nx < 1 || p->ny < 1) return 0;
-  return adj_steps_scratch_bytes(p, p->precision == LB_FP64 ? 8 : 4);
+  return p->precision == LB_FP64 ? adj_steps_scratch_bytes(p, 8, kTileY) : adj_steps_scratch_bytes(p, 4, 8);
 }
 
 int lb_adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, double* dtheta, void* scratch,
@@ -676,15 +699,16 @@ int lb_adjoint_steps(lb_handle* h, const void* const* states, int k, void* lam, 
       std::snprintf(h->err, sizeof(h->err), "lb_adjoint_steps: state %d is null", j);
       return LB_EINVAL;
     }
-  const size_t need = lb_adjoint_steps_scratch_bytes(&h->p);
+  // (The former size, partials of 16-row tiles, is enough for the kernel with those.)
+  const size_t need = adj_steps_scratch_bytes(&h->p, h->p.precision == LB_FP64 ? 8 : 4, kTileY);
   if (!scratch || scratch_bytes < need) {
     std::snprintf(h->err, sizeof(h->err), "lb_adjoint_steps needs %zu bytes of scratch, got %zu", need,
                   scratch ? scratch_bytes : 0);
     return LB_ENOMEM;
   }
   switch (h->p.precision) {
-    case LB_FP64: return adjoint_steps<double, double>(h, states, k, lam, dtheta, scratch);
-    case LB_FP32: return adjoint_steps<float, float>(h, states, k, lam, dtheta, scratch);
+    case LB_FP64: return adjoint_steps<double, double>(h, states, k, lam, dtheta, scratch, scratch_bytes);
+    case LB_FP32: return adjoint_steps<float, float>(h, states, k, lam, dtheta, scratch, scratch_bytes);
     default:
       std::snprintf(h->err, sizeof(h->err), "lb_adjoint_steps supports FP64 and FP32 storage");
       return LB_ENOTSUP;
