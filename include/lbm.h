@@ -298,8 +298,8 @@ int lb_batch_tune(lb_batch* b, int trial_steps, double* best_ms_per_step);
 int lb_batch_config(const lb_batch* b, int* tile_y, int* blocks_per_sm, int* grid);
 int lb_batch_uses_tma(const lb_batch* b);
 /* Sets the launch form by hand: shape 0, 1, 2 = plain loads with 32 x 16 tiles at
- * 64 registers, 32 x 16 at 80, 32 x 32 at 64 (blocks_per_sm 0 = one block per tile,
- * else a persistent grid); shape 3, 4 = the persistent tensor-copy kernel at 80 and
+ * 64 registers, 32 x 16 at 80, 32 x 32 at 64 (blocks_per_sm 0 = one block per tile, in
+ * shape 1 per 8-row half of a tile, else a persistent grid); shape 3, 4 = the persistent tensor-copy kernel at 80 and
  * 128 registers walking the tile list statically (block b: tiles b, b + grid, ...);
  * shape 5, 6 = the same at 80 and 128 registers taking tiles by ticket, with two
  * tiles' windows in flight per block (blocks_per_sm >= 1 for 3 - 6).  LB_EINVAL

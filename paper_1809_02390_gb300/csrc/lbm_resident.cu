@@ -70,10 +70,15 @@ bool res_plan(int nx, int ny, int precision, ResPlan* out) {
   return found;
 }
 
+// Most nodes of a resident FP32 or FP16 lattice (res_configure); FP64 lattices of that size
+// do not fit the SMs' shared memory.
+constexpr long long kResNodes = 340000;
+
 // Largest over the precisions, so that the scratch size differs between them by the
 // density plane alone.
 size_t res_mail_bytes(int nx, int ny) {
   size_t words = 0;
+  if ((long long)nx * ny > kResNodes) return 0;
   for (int precision : {int(LB_FP64), int(LB_FP32), int(LB_FP16S)}) {
     ResPlan p;
     if (res_plan(nx, ny, precision, &p) && p.words > words) words = p.words;
@@ -84,10 +89,10 @@ size_t res_mail_bytes(int nx, int ny) {
 cudaError_t res_configure(lb_handle* h, void* mail) {
   h->use_res = false;
   ResPlan p;
-  // FP32 and FP16 up to 340,000 nodes: above, a tile's pitch no longer avoids bank conflicts
+  // FP32 and FP16 up to kResNodes: above, a tile's pitch no longer avoids bank conflicts
   // and a step is no faster than a launch of k_step_fused (us: FP32 576^2 4.9 against 5.3,
   // 600^2 6.8 / 5.7; FP16 480^2 4.7 / 4.9, 576^2 6.0 / 6.3, 640 x 600 7.0 / 6.7, 800^2 10.8 / 9.8).
-  if (h->p.precision != LB_FP64 && (long long)h->p.nx * h->p.ny > 340000) return cudaSuccess;
+  if (h->p.precision != LB_FP64 && (long long)h->p.nx * h->p.ny > kResNodes) return cudaSuccess;
   if (!mail || h->variant != LB_FUSED || !res_plan(h->p.nx, h->p.ny, h->p.precision, &p)) return cudaSuccess;
   const void* k = res_kernel(h->p.precision);
   int dev = 0, coop = 0, sms = 0, per_sm = 0;
