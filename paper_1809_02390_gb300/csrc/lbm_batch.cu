@@ -661,6 +661,8 @@ int lb_batch_init(lb_batch** out, const lb_params* ps, int n, void* pool_a, void
                                        tile_kind(q * kTileX, r * kShapeTY[s], L.nx, L.ny), L.offset});
     }
   }
+  size_t interior = 0;  // tiles whose windows tensor copies deliver
+  for (const TileRec& t : h_tiles[0]) interior += t.kind == kTensorCopy;
   uintptr_t m = align(reinterpret_cast<uintptr_t>(meta));
   for (int s = 0; s < kTileLists; ++s) {
     b->d_desc[s] = reinterpret_cast<BatchLattice*>(m);
@@ -747,10 +749,13 @@ int lb_batch_init(lb_batch** out, const lb_params* ps, int n, void* pool_a, void
   // tickets and the persistent plain-load grid: 0.92 M nodes 14.4, 20.3, 24.8; 1.18 M 19.5,
   // 23.3, 27.6); larger ones: tensor copies with tiles by ticket (4.9 M nodes 71.7, half
   // tiles 73.7, the grid 101.7; 6.7 M 96.2, 101.1, 138.9).  The line lies at 100 MB of the
-  // 129 MB of L2 (1.46 M nodes), where one lattice's step changes sides.
+  // 129 MB of L2 (1.46 M nodes), where one lattice's step changes sides.  Tickets need seven
+  // tiles of ten inside their lattices, the others' windows come by per-thread copies (tickets
+  // against half tiles: 80% inside 115.5, 120.4; 76% 116.3, 119.8; 68% 116.4, 116.0; 64% 98.3,
+  // 94.9; 53% 88.8, 82.5; 42% 117.8, 103.7).
   b->shape = 1;
   b->blocks_per_sm = 0;
-  if (b->tma_ok && 2 * off * sizeof(float) > (size_t(100) << 20)) {
+  if (b->tma_ok && 2 * off * sizeof(float) > (size_t(100) << 20) && 10 * interior >= 7 * h_tiles[0].size()) {
     int mb = 1;
     if (max_blocks(b, kShapeDyn, &mb) != LB_OK) return bail(LB_ECUDA, b->err);
     b->shape = kShapeDyn;

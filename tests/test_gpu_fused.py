@@ -72,3 +72,19 @@ def test_half_tiles_of_a_batch(layout):
         assert torch.equal(b.state(i), lat.state()), s
         lat.close()
     b.close()
+
+
+@pytest.mark.parametrize("nx,ny,n,tickets", [(130, 100, 120, False), (900, 800, 3, True)])
+def test_default_form_of_a_large_pool(nx, ny, n, tickets):
+    """Above 100 MB: tickets only if most tiles lie inside their lattices."""
+    from paper_1809_02390_gb300 import Batch, Lattice
+
+    b = Batch([_rho(nx, ny)] * n, [dict(Tr=0.8) for _ in range(n)])
+    assert b.config()["tensor_copies"] == tickets
+    b.run(3)
+    lat = Lattice(_rho(nx, ny), precision="fp32", Tr=0.8)
+    lat.step(3)
+    for i in (0, n // 2, n - 1):
+        assert torch.equal(b.state(i), lat.state())
+    b.close()
+    lat.close()
