@@ -8,8 +8,8 @@
 //
 // Measured, before -> after (us a step): a step of the adjoint at 256^2 FP32 6.3 -> 5.1;
 // D2Q9 FP32 1003 x 517 11.5 -> 11.2; rows layout FP32, 20 launches, 1024^2 18.7 -> 17.1,
-// 2048^2 54.5 -> 52.5, 4096^2 192.6 -> 190.5 (the same by graph: 16.6 -> 16.4, 51.6 -> 51.5,
-// 189.5 -> 189.7); D3Q19 FP32 64^3 14.4 -> 14.2, 256^3 469 -> 458; 48 lattices of a batch
+// 2048^2 54.5 -> 52.5, 4096^2 192.6 -> 190.5 (by graph 16.6 -> 16.4, 51.6 -> 51.5, 189.5 ->
+// 189.7; these three before follow_predecessor_only); D3Q19 FP32 64^3 14.4 -> 14.2, 256^3 469 -> 458; 48 lattices of a batch
 // 76.6 -> 75.6.  It costs nothing anywhere that was tried, so every step kernel is
 // launched so, except into a caller's own capture.
 #pragma once
@@ -27,6 +27,12 @@ namespace lbm {
 __device__ __forceinline__ void follow_predecessor() {
   asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// The same without the early start of the successor, whose blocks then come up as this
+// kernel's exit: for persistent kernels, where they would hold the SMs' free slots while
+// tiles are left (20 steps, against an ordinary launch and an early start: FP32 4096^2 3738,
+// 3704 -> 3689 us; FP16 4096 x 2048 2009, 1972 -> 1962).
+__device__ __forceinline__ void follow_predecessor_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // overlap = false: an ordinary launch (a caller's stream capture records plain edges).
 template <typename... P, typename... A>
