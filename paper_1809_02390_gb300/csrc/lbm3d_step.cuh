@@ -239,9 +239,7 @@ __device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9],
   const V JZ = fmav(c.nquarter, oz, c.eighth * (jz + Fz));
   const V mx = c.om8 * (D12p - D13p), my = c.om8 * (D23p - D12m), mz = c.om8 * (D13m - D23m);
 
-  // Inverse transform.  o[0] takes what the other populations' even parts leave of the
-  // mass, so that the rounding of their constants does not shift it step by step (200
-  // FP32 steps of 64^3: 3e-6 off 64 bits with o[0] from T and a, 5e-7 with this).
+  // Inverse transform.
   const V a6 = c.sixth * as;
   const V ev0 = fmav(c.sixth, Xas, a6), et = fmav(c.n12, Xas, a6);
   const V ev1 = fmav(c.quarter, Was, et), ev2 = fmav(c.nquarter, Was, et);
@@ -250,7 +248,6 @@ __device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9],
   o[5] = ev2 + oz, o[6] = ev2 - oz;
   const V ce = c.i24 * (Ts - as);
   const V cx = fmav(c.i24, Xes, ce), eyz = fmav(c.n12, Xes, ce);
-  o[0] = fmav(c.n4, fmav(c.two, cx, eyz), fmav(c.n2, fmav(c.two, et, ev0), delta));
   const V w8 = c.eighth * Wes;
   const V exy = cx + w8, exz = cx - w8;
   auto edge = [&](V e, V p, V odp, V odm, V& o1, V& o2, V& o3, V& o4) {
@@ -261,6 +258,22 @@ __device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9],
   edge(exy, xy, (JX + JY) + (mx - my), (JX - JY) + (mx + my), o[7], o[8], o[9], o[10]);
   edge(exz, xz, (JX + JZ) - (mx - mz), (JX - JZ) - (mx + mz), o[11], o[12], o[13], o[14]);
   edge(eyz, yz, (JY + JZ) + (my - mz), (JY - JZ) + (my + mz), o[15], o[16], o[17], o[18]);
+  // o[0] takes what the others leave of the mass.  FP32: of the populations as they are
+  // stored, one pair after the other.  Taking their even parts before the last rounding
+  // (e + p + od) instead leaves that rounding out, which in quiet liquid and gas is the
+  // same every step: 2e-9 of the mass lost a step, 1.3e-6 off 64 bits after 400 steps of
+  // two-phase 24^3 lattices, against 2e-11 and 4e-7 with the stored ones (collide3_moments:
+  // 2e-10 and 6e-7); summing the 18 first and taking them off at once leaves 1e-10 a step.
+  // FP64 has no such drift to speak of (1e-18 a step) and its pipe no room for 14
+  // instructions more.
+  if constexpr (Val<V>::lanes == 2) {
+    V t = delta;
+#pragma unroll
+    for (int P = 0; P < 9; ++P) t = t - (o[2 * P + 1] + o[2 * P + 2]);
+    o[0] = t;
+  } else {
+    o[0] = fmav(c.n4, fmav(c.two, cx, eyz), fmav(c.n2, fmav(c.two, et, ev0), delta));
+  }
 }
 
 // 12 times the force stencil sum_i omega_i rho(x + e_i) e_i (Eq. 12) from the density
