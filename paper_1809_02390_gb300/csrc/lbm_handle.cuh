@@ -56,7 +56,6 @@ struct lb_handle {
   bool forced_blocks, forced_walk;  // lb_set_step_blocks, lb_set_tile_dispatch fixed another launch form
   lbm::ResPlan res;
   void* res_mail;         // exchange words (end of the scratch buffer)
-  unsigned res_epoch;     // numbers up to this one have been used
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
   bool overlap;           // the steps' launches may overlap their predecessor's end (lbm_launch.cuh)
   int graph_k;            // while capturing: the place of the launch in the graph (else -1)
@@ -83,8 +82,8 @@ bool encode_volume_map(CUtensorMap* map, const void* base, int nx, int ny, int n
 bool res_plan(int nx, int ny, int precision, ResPlan* out);
 // Bytes of the exchange buffer (0 when no precision of this size runs resident).
 size_t res_mail_bytes(int nx, int ny);
-// Decides whether the handle can run resident and clears the exchange buffer `mail`
-// (device memory of res_mail_bytes, 16-byte aligned, or null).
+// Decides whether the handle can run resident with the exchange buffer `mail` (device
+// memory of res_mail_bytes, 16-byte aligned, or null; its contents do not matter).
 cudaError_t res_configure(lb_handle* h, void* mail);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
 // null): device memory that receives the states after every `every` (< 2^31) steps.

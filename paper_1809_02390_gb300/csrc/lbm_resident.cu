@@ -104,11 +104,8 @@ cudaError_t res_configure(lb_handle* h, void* mail) {
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, p.threads, p.smem);
   if (e != cudaSuccess) return e;
   if (!coop || per_sm < 1 || sms < p.gx * p.gy) return cudaSuccess;
-  e = cudaMemsetAsync(mail, 0, 2 * p.words * sizeof(uint4), h->stream);
-  if (e != cudaSuccess) return e;
   h->res = p;
   h->res_mail = mail;
-  h->res_epoch = 0;
   h->use_res = true;
   return cudaSuccess;
 }
@@ -127,7 +124,6 @@ cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout,
                rec_every,
                static_cast<uint4*>(h->res_mail),
                h->wait_error,
-               h->res_epoch,
                unsigned(h->steps),
                nsteps,
                h->p.nx,
@@ -154,11 +150,6 @@ cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
   while (nsteps > 0) {
     // Never a launch of one step: it could not write its result in place.
     int64_t n = nsteps <= kResChunk ? nsteps : (nsteps == kResChunk + 1 ? kResChunk - 2 : kResChunk);
-    if (h->res_epoch > 0xf0000000u) {
-      const cudaError_t e = cudaMemsetAsync(h->res_mail, 0, 2 * h->res.words * sizeof(uint4), h->stream);
-      if (e != cudaSuccess) return e;
-      h->res_epoch = 0;
-    }
     const void* in = h->f[h->cur];
     void* out = h->f[n & 1 ? 1 - h->cur : h->cur];
     cudaError_t e;
@@ -173,7 +164,6 @@ cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
       rec = static_cast<char*>(rec) + size_t(states) * lb_state_bytes(&h->p);
       first = states ? every - (n - first) % every : first - n;
     }
-    h->res_epoch += unsigned(n);
     h->steps += n;
     if (n & 1) h->cur = 1 - h->cur;
     nsteps -= n;

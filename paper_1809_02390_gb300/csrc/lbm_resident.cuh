@@ -27,7 +27,16 @@
 // column groups of the diagonal tiles.  Words are double-buffered by the parity of
 // the step: a tile writes step s + 2 only after reading every neighbour's step
 // s + 1, which that neighbour sent after it had read step s.
+//
+// What the scratch buffer held before a run is never taken for a word of it: every tile
+// clears its own words first, and no tile reads any before all tiles have (a grid barrier,
+// arrived at right after clearing and waited for a whole step later, so that its trip is
+// hidden).  So handles that share a scratch buffer may run in turn, whatever they left in it.
 #pragma once
+
+#include <cooperative_groups.h>
+
+#include <utility>
 
 #include "lbm_tma.cuh"
 
@@ -119,7 +128,6 @@ struct ResArgs {
   int rec_first, rec_every;
   uint4* mail;         // exchange words, two parities
   int* err;
-  unsigned epoch;      // step s carries the number epoch + s + 1
   unsigned step0;      // time step number of step 0 (seeds the FP16 rounding)
   int nsteps, nx, ny, gx, gy, wmax, hmax, pitch;
   int stochastic;
@@ -330,8 +338,19 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
   real* rho = reinterpret_cast<real*>(dyn + res_table_bytes(a.wmax, a.hmax, L));
   S* cur = reinterpret_cast<S*>(rho + plane);
   S* nxt = cur + 9 * plane;
-  const size_t mail_stride = size_t(a.gx) * a.gy * 6 * (a.hmax + a.wmax) * ResTraits<S>::words;
+  constexpr int W = ResTraits<S>::words;
+  const int own_words = 6 * (a.hmax + a.wmax) * W;  // of a tile, one parity
+  const size_t mail_stride = size_t(a.gx) * a.gy * own_words;
 
+  // This tile's words: number 0, which no step carries.  The barrier cannot block: the
+  // launch is cooperative, and every block arrives before it waits for anything.
+  for (int q = tid; q < 2 * own_words; q += T) {
+    const bool odd = q >= own_words;
+    st_word(a.mail + (odd ? mail_stride : 0) + size_t(blockIdx.x) * own_words + (q - (odd ? own_words : 0)),
+            make_uint4(0u, 0u, 0u, 0u));
+  }
+  const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  auto cleared = grid.barrier_arrive();
   // Initial state of tile and halo (periodic), and the tables.
   for (int q = tid; q < (w + 4) * (h + 4); q += T) {
     const int ly = q / (w + 4), lx = q - ly * (w + 4);
@@ -394,12 +413,12 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
   __syncthreads();
   for (int q = inner_begin; q < sl.total; q += T) density(cur, q);  // phase 1a of step 0
 
-  constexpr int W = ResTraits<S>::words;
   S* rec = a.rec;
   int until = a.rec_first;  // steps until the next recorded state
   for (int s = 0;; ++s) {
-    const unsigned number = a.epoch + unsigned(s);
+    const unsigned number = unsigned(s);  // of the words read; step s sends s + 1
     bool late = false;
+    if (s == 1) grid.barrier_wait(std::move(cleared));
     if (s > 0) {
       // Two groups of this thread at a time; the first two are asked for before the
       // densities of the inner nodes, which hide the trip through L2.
