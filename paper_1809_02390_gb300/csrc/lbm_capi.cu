@@ -836,12 +836,12 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
     capture = cudaStreamCaptureStatusActive;
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_record(h) && capture == cudaStreamCaptureStatusNone) {
+  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_record(h) && capture == cudaStreamCaptureStatusNone &&
+      record_by_elements(h->p, reinterpret_cast<uintptr_t>(at))) {
     LB_CUDA(h, res_run(h, nsteps, states, every));
     return LB_OK;
   }
-  const bool aligned = reinterpret_cast<uintptr_t>(at) % 16 == 0 && bytes % 16 == 0;
-  if (every == 1 && (aligned || !h->use_tma)) {
+  if (every == 1 && record_in_place(h->p, reinterpret_cast<uintptr_t>(at), bytes, h->use_tma)) {
     // Every state is wanted: step from each straight into the next (the handle's buffers
     // stand aside), and bring the last one home.
     void* const f[2] = {h->f[0], h->f[1]};
