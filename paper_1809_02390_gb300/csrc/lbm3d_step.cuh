@@ -747,25 +747,25 @@ __device__ __forceinline__ void pull19(const T* __restrict__ f, S N, int nx, int
   const int r0m = (zm * ny + y) * nx, r0p = (zp * ny + y) * nx;
   const int rmm = (zm * ny + ym) * nx, rpp = (zp * ny + yp) * nx;
   const int rmp = (zp * ny + ym) * nx, rpm = (zm * ny + yp) * nx;
-  v[0] = __ldg(f + r00 + x);
-  v[1] = __ldg(f + N + r00 + xm);
-  v[2] = __ldg(f + 2 * N + r00 + xp);
-  v[3] = __ldg(f + 3 * N + rm0 + x);
-  v[4] = __ldg(f + 4 * N + rp0 + x);
-  v[5] = __ldg(f + 5 * N + r0m + x);
-  v[6] = __ldg(f + 6 * N + r0p + x);
-  v[7] = __ldg(f + 7 * N + rm0 + xm);
-  v[8] = __ldg(f + 8 * N + rp0 + xp);
-  v[9] = __ldg(f + 9 * N + rp0 + xm);
-  v[10] = __ldg(f + 10 * N + rm0 + xp);
-  v[11] = __ldg(f + 11 * N + r0m + xm);
-  v[12] = __ldg(f + 12 * N + r0p + xp);
-  v[13] = __ldg(f + 13 * N + r0p + xm);
-  v[14] = __ldg(f + 14 * N + r0m + xp);
-  v[15] = __ldg(f + 15 * N + rmm + x);
-  v[16] = __ldg(f + 16 * N + rpp + x);
-  v[17] = __ldg(f + 17 * N + rmp + x);
-  v[18] = __ldg(f + 18 * N + rpm + x);
+  v[0] = lbm::ld_st(f + r00 + x);
+  v[1] = lbm::ld_st(f + N + r00 + xm);
+  v[2] = lbm::ld_st(f + 2 * N + r00 + xp);
+  v[3] = lbm::ld_st(f + 3 * N + rm0 + x);
+  v[4] = lbm::ld_st(f + 4 * N + rp0 + x);
+  v[5] = lbm::ld_st(f + 5 * N + r0m + x);
+  v[6] = lbm::ld_st(f + 6 * N + r0p + x);
+  v[7] = lbm::ld_st(f + 7 * N + rm0 + xm);
+  v[8] = lbm::ld_st(f + 8 * N + rp0 + xp);
+  v[9] = lbm::ld_st(f + 9 * N + rp0 + xm);
+  v[10] = lbm::ld_st(f + 10 * N + rm0 + xp);
+  v[11] = lbm::ld_st(f + 11 * N + r0m + xm);
+  v[12] = lbm::ld_st(f + 12 * N + r0p + xp);
+  v[13] = lbm::ld_st(f + 13 * N + r0p + xm);
+  v[14] = lbm::ld_st(f + 14 * N + r0m + xp);
+  v[15] = lbm::ld_st(f + 15 * N + rmm + x);
+  v[16] = lbm::ld_st(f + 16 * N + rpp + x);
+  v[17] = lbm::ld_st(f + 17 * N + rmp + x);
+  v[18] = lbm::ld_st(f + 18 * N + rpm + x);
 }
 
 template <typename T>

@@ -307,15 +307,15 @@ __global__ void __launch_bounds__(adj_threads<TY, ROWS>, adj_min_blocks<real, TY
     } else {
       const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
       const int oc = gy * nx, om = ym * nx, op = yp * nx;
-      mu9[0] = mu_in[off];
-      mu9[1] = mu_in[plane + oc + xp];
-      mu9[2] = mu_in[2 * plane + op + gx];
-      mu9[3] = mu_in[3 * plane + oc + xm];
-      mu9[4] = mu_in[4 * plane + om + gx];
-      mu9[5] = mu_in[5 * plane + op + xp];
-      mu9[6] = mu_in[6 * plane + op + xm];
-      mu9[7] = mu_in[7 * plane + om + xm];
-      mu9[8] = mu_in[8 * plane + om + xp];
+      mu9[0] = ld_st(mu_in + (off));
+      mu9[1] = ld_st(mu_in + (plane + oc + xp));
+      mu9[2] = ld_st(mu_in + (2 * plane + op + gx));
+      mu9[3] = ld_st(mu_in + (3 * plane + oc + xm));
+      mu9[4] = ld_st(mu_in + (4 * plane + om + gx));
+      mu9[5] = ld_st(mu_in + (5 * plane + op + xp));
+      mu9[6] = ld_st(mu_in + (6 * plane + op + xm));
+      mu9[7] = ld_st(mu_in + (7 * plane + om + xm));
+      mu9[8] = ld_st(mu_in + (8 * plane + om + xp));
     }
     real ob[9];
     ob[0] = mu9[0] + rb[ly][lx];
