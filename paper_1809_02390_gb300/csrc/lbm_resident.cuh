@@ -30,8 +30,8 @@
 //
 // What the scratch buffer held before a run is never taken for a word of it: every tile
 // clears its own words first, and no tile reads any before all tiles have (a grid barrier,
-// arrived at right after clearing and waited for a whole step later, so that its trip is
-// hidden).  So handles that share a scratch buffer may run in turn, whatever they left in it.
+// arrived at right after clearing and waited for once the tile is loaded; waiting in the
+// second step instead kept its state alive in the loop, 2.17 us a step at 256^2).  So handles that share a scratch buffer may run in turn, whatever they left in it.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -412,13 +412,13 @@ __global__ void __launch_bounds__(ResTraits<S>::max_threads, 1) k_resident(const
   for (int k = 0; k < warps; ++k) gate_threads += k < edge_warps || (k & 3) < shared ? 32 : 0;
   __syncthreads();
   for (int q = inner_begin; q < sl.total; q += T) density(cur, q);  // phase 1a of step 0
+  grid.barrier_wait(std::move(cleared));
 
   S* rec = a.rec;
   int until = a.rec_first;  // steps until the next recorded state
   for (int s = 0;; ++s) {
     const unsigned number = unsigned(s);  // of the words read; step s sends s + 1
     bool late = false;
-    if (s == 1) grid.barrier_wait(std::move(cleared));
     if (s > 0) {
       // Two groups of this thread at a time; the first two are asked for before the
       // densities of the inner nodes, which hide the trip through L2.
