@@ -162,7 +162,7 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
  * nodes) takes calls of several steps (at least 4, FP32 and FP16 12) in one cooperative
  * launch that keeps it in the SMs' shared memory (same bits; waits between its blocks are
  * bounded at 10 s and reported by lb_status), unless lb_set_step_blocks or
- * lb_set_tile_dispatch ask for another form.  Else runs of 64 steps replay a CUDA graph that the handle captures on
+ * lb_set_tile_dispatch asked for a tensor-copy form (lb_step_form tells which form serves a call).  Else runs of 64 steps replay a CUDA graph that the handle captures on
  * first use (again after lb_set_step_blocks or lb_set_tile_dispatch change the
  * launch); the graph runs on a stream the handle owns, ordered after the caller's
  * stream's earlier work and before its later work, and gives the same bits as 64
@@ -380,6 +380,18 @@ int lb_uses_tma(const lb_handle* h);
  * 1 when the step does not use tensor copies or the handle has no scratch. */
 int lb_set_tile_dispatch(lb_handle* h, int dynamic);
 int lb_tile_dispatch(const lb_handle* h);
+
+/* The form that lb_step(h, nsteps) takes outside a stream capture: the two-pass variant,
+ * the fused step by plain loads, by tensor copies with tiles walked statically or taken by
+ * ticket, or all steps in one resident launch.  LB_EINVAL for a null handle or nsteps < 1. */
+enum lb_step_kind {
+  LB_STEP_TWO_PASS = 0,
+  LB_STEP_PLAIN = 1,
+  LB_STEP_TENSOR_WALK = 2,
+  LB_STEP_TENSOR_TICKETS = 3,
+  LB_STEP_RESIDENT = 4
+};
+int lb_step_form(const lb_handle* h, int64_t nsteps);
 
 /* Measurement aid (no counterpart in the paper): one pass with the step's memory
  * traffic and none of its arithmetic, a copy of the state into the other buffer

@@ -58,6 +58,7 @@ SIGNATURES = [
     ("lb_init", ctypes.c_int, [ctypes.POINTER(_V), _P, _V, _V, _V, ctypes.c_size_t, _V, ctypes.c_int, _V]),
     ("lb_step", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_step_record", ctypes.c_int, [_V, ctypes.c_int64, ctypes.c_int64, _V]),
+    ("lb_step_form", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_state", _V, [_V]),
     ("lb_steps_done", ctypes.c_int64, [_V]),
     ("lb_moments", ctypes.c_int, [_V, _V, _V, _V]),
@@ -182,6 +183,17 @@ def lb_step(h: int, nsteps: int) -> None:
 
 def lb_step_record(h: int, nsteps: int, every: int, states: int) -> None:
     check(lib().lb_step_record(h, int(nsteps), int(every), states), h)
+
+
+# Forms of a step call (enum lb_step_kind).
+LB_STEP_TWO_PASS, LB_STEP_PLAIN, LB_STEP_TENSOR_WALK, LB_STEP_TENSOR_TICKETS, LB_STEP_RESIDENT = range(5)
+
+
+def lb_step_form(h: int, nsteps: int) -> int:
+    form = lib().lb_step_form(h, int(nsteps))
+    if form < 0:
+        raise LBError(form, "lb_step_form: null handle or nsteps < 1")
+    return form
 
 
 def lb_state(h: int) -> int:

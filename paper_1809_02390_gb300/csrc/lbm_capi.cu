@@ -195,10 +195,24 @@ constexpr size_t kQueueBytes = 256;  // tile tickets of the dynamic tensor-copy 
 // steps are then launched one by one).
 size_t base_scratch_bytes(const lb_params* p) { return rho_plane_bytes(p) + reduce_bytes() + kQueueBytes; }
 
-// Whether steps take the tensor-copy kernel: h->use_tma, unless the lattice is small
-// enough for the plain one and no launch form was asked for.
-bool tensor_step(const lb_handle* h) {
-  return h->use_tma && (!h->plain_small || h->forced_blocks || h->forced_dispatch);
+// Fewest steps of a call that run resident: the launch costs some 8 us more than an
+// ordinary one (load, store, cooperative start), a step less (FP32 256^2 2.15 against 2.74 us,
+// 400^2 3.0 / 4.2, FP16 256^2 2.5 / 3.35: from 12 or 13, 8 and 8 steps; FP64 64^2 7.6 / 21.5).
+int64_t res_min_steps(const lb_handle* h) { return h->p.precision == LB_FP64 ? 4 : 12; }
+// The same for runs that record states.
+int64_t res_min_record(const lb_handle* h) { return h->p.precision == LB_FP64 ? 2 : 12; }
+
+// The form of a single launch (enum lb_step_kind): tensor copies where the handle can, unless
+// the lattice is small enough for the plain kernel and no tensor-copy form was asked for.
+int launch_form(const lb_handle* h) {
+  if (h->variant != LB_FUSED) return LB_STEP_TWO_PASS;
+  if (!h->use_tma || (h->plain_small && !h->forced_blocks && !h->forced_dispatch)) return LB_STEP_PLAIN;
+  return h->use_dyn ? LB_STEP_TENSOR_TICKETS : LB_STEP_TENSOR_WALK;
+}
+
+// Whether a call of nsteps steps runs resident (outside a capture).
+bool resident_call(const lb_handle* h, int64_t nsteps, int64_t least) {
+  return h->use_res && !h->forced_blocks && !h->forced_dispatch && nsteps >= least;
 }
 
 template <typename V, typename real, typename store_t>
@@ -213,15 +227,16 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
     rnd.step = h->step_word;
     rnd.k = h->graph_k;
   }
-  if (h->variant == LB_FUSED) {
+  const int form = launch_form(h);
+  if (form != LB_STEP_TWO_PASS) {
     const dim3 grd((nx + kTileX - 1) / kTileX, (ny + kFusedRows - 1) / kFusedRows);
     if constexpr (sizeof(store_t) <= 4 && std::is_same<V, f2>::value) {
-      if (tensor_step(h) && h->use_dyn) {
+      if (form == LB_STEP_TENSOR_TICKETS) {
         launch_step_kernel(h->overlap, k_step_tma_dyn<V, store_t>, h->dyn_grid, kFusedThreads, Win2<store_t>::smem,
                            h->stream, h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd, h->queue);
         return;
       }
-      if (tensor_step(h)) {
+      if (form == LB_STEP_TENSOR_WALK) {
         k_step_tma<V, store_t, false><<<h->tma_grid, kFusedThreads, Win<store_t>::smem, h->stream>>>(
             h->tmap[h->cur], fin, fout, nx, ny, h->st, cv, h->wait_error, rnd);
         return;
@@ -707,12 +722,6 @@ namespace {
 
 // Steps per captured graph (even, so a replay ends on the buffer it started from).
 constexpr int kStepGraph = 64;
-// Fewest steps of a call that run resident: the launch costs some 8 us more than an
-// ordinary one (load, store, cooperative start), a step less (FP32 256^2 2.15 against 2.74 us,
-// 400^2 3.0 / 4.2, FP16 256^2 2.5 / 3.35: from 12 or 13, 8 and 8 steps; FP64 64^2 7.6 / 21.5).
-int64_t res_min_steps(const lb_handle* h) { return h->p.precision == LB_FP64 ? 4 : 12; }
-// The same for runs that record states.
-int64_t res_min_record(const lb_handle* h) { return h->p.precision == LB_FP64 ? 2 : 12; }
 
 void launch_one_step(lb_handle* h) {
   switch (h->p.precision) {
@@ -724,8 +733,7 @@ void launch_one_step(lb_handle* h) {
 
 // The launch configuration a graph bakes in: kernel form and grid sizes.
 long long step_config(const lb_handle* h) {
-  return (long long)h->variant | ((long long)tensor_step(h) << 2) | ((long long)h->use_dyn << 3) |
-         ((long long)h->tma_grid << 4) | ((long long)h->dyn_grid << 34);
+  return (long long)launch_form(h) | ((long long)h->tma_grid << 4) | ((long long)h->dyn_grid << 34);
 }
 
 // Captures (once per starting buffer and configuration) kStepGraph steps into a
@@ -789,7 +797,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_steps(h) && capture == cudaStreamCaptureStatusNone) {
+  if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_steps(h))) {
     LB_CUDA(h, res_run(h, nsteps, nullptr, 1));
     return LB_OK;
   }
@@ -836,7 +844,7 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
     capture = cudaStreamCaptureStatusActive;
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (h->use_res && !h->forced_blocks && !h->forced_walk && nsteps >= res_min_record(h) && capture == cudaStreamCaptureStatusNone &&
+  if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_record(h)) &&
       record_by_elements(h->p, reinterpret_cast<uintptr_t>(at))) {
     LB_CUDA(h, res_run(h, nsteps, states, every));
     return LB_OK;
@@ -1031,9 +1039,13 @@ int lb_set_tile_dispatch(lb_handle* h, int dynamic) {
   if (dynamic && !(h->use_tma && h->queue))
     return fail(h, LB_ENOTSUP, "dynamic dispatch needs the tensor-copy step and the scratch buffer");
   h->use_dyn = dynamic != 0;
-  h->forced_walk = h->use_tma && !dynamic;
-  h->forced_dispatch = true;
+  h->forced_dispatch = h->use_tma;
   return LB_OK;
+}
+
+int lb_step_form(const lb_handle* h, int64_t nsteps) {
+  if (!h || nsteps < 1) return LB_EINVAL;
+  return resident_call(h, nsteps, res_min_steps(h)) ? LB_STEP_RESIDENT : launch_form(h);
 }
 
 int lb_tile_dispatch(const lb_handle* h) { return h && h->use_tma && h->use_dyn ? 1 : 0; }

@@ -52,8 +52,8 @@ struct lb_handle {
   // shared memory.
   bool use_res;
   bool plain_small;       // small enough for k_step_fused although tensor copies could serve it
-  bool forced_dispatch;   // lb_set_tile_dispatch was called
-  bool forced_blocks, forced_walk;  // lb_set_step_blocks, lb_set_tile_dispatch fixed another launch form
+  bool forced_dispatch;   // lb_set_tile_dispatch asked for a tensor-copy form
+  bool forced_blocks;     // lb_set_step_blocks fixed its grid
   lbm::ResPlan res;
   void* res_mail;         // exchange words (end of the scratch buffer)
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
