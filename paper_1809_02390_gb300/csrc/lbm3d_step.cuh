@@ -360,7 +360,7 @@ __host__ __device__ __forceinline__ bool tensor_tile(int x0, int y0, int nx, int
 // number of blocks and stages, at 38.6 without the halo, and at 39.1 with tensor copies.
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(Win3<T>::threads, d3_blocks<T>())
-    k_d3_step(const T* __restrict__ fin, T* __restrict__ fout, int nx, int ny, int nz, int tw_, int th_, int tz,
+    k_d3_step(const T* fin, T* __restrict__ fout, int nx, int ny, int nz, int tw_, int th_, int tz,
               const CV3<typename ValOf<T>::V> c, const __grid_constant__ CUtensorMap map, int have_map, int* __restrict__ err) {
   using V = typename ValOf<T>::V;
   using W = Win3<T>;
@@ -741,7 +741,7 @@ __device__ __forceinline__ void collide3_moments(const C3<T>& c, const T* f, T d
 // the stride between population planes, in the type S of the plane offsets (int
 // when 19 N < 2^31, else long long; node indices are int).
 template <typename T, typename S>
-__device__ __forceinline__ void pull19(const T* __restrict__ f, S N, int nx, int ny, int xm, int x, int xp, int ym,
+__device__ __forceinline__ void pull19(const T* f, S N, int nx, int ny, int xm, int x, int xp, int ym,
                                        int y, int yp, int zm, int z, int zp, T* v) {
   const int r00 = (z * ny + y) * nx, rm0 = (z * ny + ym) * nx, rp0 = (z * ny + yp) * nx;
   const int r0m = (zm * ny + y) * nx, r0p = (zp * ny + y) * nx;
@@ -803,7 +803,7 @@ __device__ __forceinline__ void stencil_collide_store(const C3<T>& c, const T (*
 // S: type of the plane offsets (int when 19 nx ny nz < 2^31, else long long).
 template <typename S>
 __global__ void __launch_bounds__(TX* kPullTY, 3)
-    k_d3_pull(const float* __restrict__ fin, float* __restrict__ fout, int nx, int ny, int nz, int tz, C3<float> c) {
+    k_d3_pull(const float* fin, float* __restrict__ fout, int nx, int ny, int nz, int tz, C3<float> c) {
   using T = float;
   lbm::follow_predecessor();
   __shared__ T pl[3][kPullHY][HX];

@@ -196,7 +196,7 @@ constexpr int adj_min_blocks() {
 
 template <typename real, typename store_t, int TY, int ROWS>
 __global__ void __launch_bounds__(adj_threads<TY, ROWS>, adj_min_blocks<real, TY, ROWS>())
-    k_adj_fused(const store_t* __restrict__ s, const real* __restrict__ mu_in, const real* __restrict__ sb_in,
+    k_adj_fused(const store_t* s, const real* mu_in, const real* sb_in,
                 real* __restrict__ mu, real* __restrict__ sbar, double* __restrict__ partial, int accumulate, int nx,
                 int ny, VCoef<real> c) {
   constexpr int NT = adj_threads<TY, ROWS>;
@@ -307,15 +307,15 @@ __global__ void __launch_bounds__(adj_threads<TY, ROWS>, adj_min_blocks<real, TY
     } else {
       const int ym = gy == 0 ? ny - 1 : gy - 1, yp = gy == ny - 1 ? 0 : gy + 1;
       const int oc = gy * nx, om = ym * nx, op = yp * nx;
-      mu9[0] = ld_st(mu_in + (off));
-      mu9[1] = ld_st(mu_in + (plane + oc + xp));
-      mu9[2] = ld_st(mu_in + (2 * plane + op + gx));
-      mu9[3] = ld_st(mu_in + (3 * plane + oc + xm));
-      mu9[4] = ld_st(mu_in + (4 * plane + om + gx));
-      mu9[5] = ld_st(mu_in + (5 * plane + op + xp));
-      mu9[6] = ld_st(mu_in + (6 * plane + op + xm));
-      mu9[7] = ld_st(mu_in + (7 * plane + om + xm));
-      mu9[8] = ld_st(mu_in + (8 * plane + om + xp));
+      mu9[0] = mu_in[off];
+      mu9[1] = mu_in[plane + oc + xp];
+      mu9[2] = mu_in[2 * plane + op + gx];
+      mu9[3] = mu_in[3 * plane + oc + xm];
+      mu9[4] = mu_in[4 * plane + om + gx];
+      mu9[5] = mu_in[5 * plane + op + xp];
+      mu9[6] = mu_in[6 * plane + op + xm];
+      mu9[7] = mu_in[7 * plane + om + xm];
+      mu9[8] = mu_in[8 * plane + om + xp];
     }
     real ob[9];
     ob[0] = mu9[0] + rb[ly][lx];
@@ -380,8 +380,8 @@ static_assert((kAdjMuOff * 4) % 128 == 0 && (kMuPlane * 4) % 128 == 0 && (kAdjSb
 
 // All threads: the staging of a wrapping tile (lattice of at least 40 x 18) by
 // per-thread asynchronous copies; commits one group.
-__device__ __forceinline__ void stage_adj_async(float* base, const float* __restrict__ s,
-                                                const float* __restrict__ mu_in, const float* __restrict__ sb_in,
+__device__ __forceinline__ void stage_adj_async(float* base, const float* s,
+                                                const float* mu_in, const float* sb_in,
                                                 int nx, int ny, int x0, int y0) {
   const int plane = nx * ny;
   for (int e = threadIdx.x; e < 9 * kMuPlane; e += kAdjThreads) {
@@ -402,8 +402,8 @@ __device__ __forceinline__ void stage_adj_async(float* base, const float* __rest
 // tensor copies that gives up sets *err (reported by lb_status) and ends the block.
 __global__ void __launch_bounds__(kAdjThreads, 3)
     k_adj_tma(const __grid_constant__ CUtensorMap tstate, const __grid_constant__ CUtensorMap tmu,
-              const __grid_constant__ CUtensorMap tsb, const float* __restrict__ s, const float* __restrict__ mu_in,
-              const float* __restrict__ sb_in, float* __restrict__ mu, float* __restrict__ sbar,
+              const __grid_constant__ CUtensorMap tsb, const float* s, const float* mu_in,
+              const float* sb_in, float* __restrict__ mu, float* __restrict__ sbar,
               double* __restrict__ partial, int accumulate, int nx, int ny, VCoef<float> c, int* __restrict__ err) {
   follow_predecessor();
   extern __shared__ __align__(128) unsigned char dyn[];

@@ -89,7 +89,7 @@ struct StoreCoef {
 
 template <typename store_t, int TY, int MINB, bool PERSIST>
 __global__ void __launch_bounds__(TileShape<TY>::threads, MINB)
-    k_step_batch(const store_t* __restrict__ pool_in, store_t* __restrict__ pool_out,
+    k_step_batch(const store_t* pool_in, store_t* __restrict__ pool_out,
                  const TileRec* __restrict__ tiles, const LatCoef<f2>* __restrict__ coef, int total_tiles,
                  VCoef<f2> common, int rows) {
   static_assert(kCoefWords <= TileShape<TY>::threads, "one coefficient word per thread");
@@ -145,7 +145,7 @@ static_assert(sizeof(LatCoef<f2>) % 16 == 0, "bulk copies move multiples of 16 b
 
 template <int MINB>
 __global__ void __launch_bounds__(kFusedThreads, MINB)
-    k_step_batch_tma(const float* __restrict__ pool_in, float* __restrict__ pool_out,
+    k_step_batch_tma(const float* pool_in, float* __restrict__ pool_out,
                      const TileRec* __restrict__ tiles, const LatCoef<f2>* __restrict__ coef,
                      const CUtensorMap* __restrict__ maps, int total_tiles, VCoef<f2> common, int* __restrict__ err,
                      int rows) {
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kFusedThreads, MINB)
 // k's.  A wait that gives up sets *err.
 template <int MINB>
 __global__ void __launch_bounds__(kFusedThreads, MINB)
-    k_step_batch_tma_dyn(const float* __restrict__ pool_in, float* __restrict__ pool_out,
+    k_step_batch_tma_dyn(const float* pool_in, float* __restrict__ pool_out,
                          const TileRec* __restrict__ tiles, const LatCoef<f2>* __restrict__ coef,
                          const CUtensorMap* __restrict__ maps, int total_tiles, VCoef<f2> common,
                          int* __restrict__ err, unsigned* __restrict__ queue, int rows) {

@@ -86,27 +86,16 @@ struct LaneType<f2> {
   using type = float;
 };
 
-// Storage <-> compute conversions.  Populations are read by ordinary global loads, not
-// through the read-only path: a step launched over its predecessor's end (lbm_launch.cuh)
-// lives while its input is still being written, and ld.global.nc (__ldg, or any load that
-// the compiler turns into one because of const __restrict__) is for data that does not
-// change while the kernel runs, waiting included.  volatile keeps these loads behind the
-// wait.
-__device__ __forceinline__ float ld_st(const float* p) {
-  float v;
-  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
-  return v;
-}
-__device__ __forceinline__ double ld_st(const double* p) {
-  double v;
-  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
-  return v;
-}
-__device__ __forceinline__ float ld_st(const __half* p) {
-  unsigned short v;
-  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(__cvta_generic_to_global(p)));
-  return __half2float(__ushort_as_half(v));
-}
+// Storage <-> compute conversions.  A step launched over its predecessor's end (lbm_launch.cuh)
+// lives while its input is still being written, so it must not read populations through the
+// read-only path (ld.global.nc: __ldg, or any load that the compiler turns into one because
+// its pointer is a const __restrict__ parameter): that is for data that does not change while
+// the kernel runs, waiting included.  Plain loads from parameters without __restrict__ stay
+// ordinary and behind the wait, a barrier for all memory (asm volatile loads, whose order is
+// fixed among themselves too, were 2% slower in the batched step).
+__device__ __forceinline__ float ld_st(const float* p) { return *p; }
+__device__ __forceinline__ double ld_st(const double* p) { return *p; }
+__device__ __forceinline__ float ld_st(const __half* p) { return __half2float(*p); }
 __device__ __forceinline__ void st_st(float* p, float v) { *p = v; }
 __device__ __forceinline__ void st_st(double* p, double v) { *p = v; }
 __device__ __forceinline__ void st_st(__half* p, float v) { *p = __float2half_rn(v); }

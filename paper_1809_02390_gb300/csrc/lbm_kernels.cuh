@@ -35,7 +35,7 @@ __device__ __forceinline__ int wrap1(int v, int n) { return v < 0 ? v + n : (v >
 // the population and row strides in elements (Strides ps, rs).  32-bit offsets:
 // the library limits the buffer to below 2^31 elements.
 template <typename real, typename store_t>
-__device__ __forceinline__ void pull_row(const store_t* __restrict__ fin, int plane, int sx, int ny, int r, int cm,
+__device__ __forceinline__ void pull_row(const store_t* fin, int plane, int sx, int ny, int r, int cm,
                                          int cc, int cp, real (&f)[9]) {
   const int rm = r == 0 ? ny - 1 : r - 1, rp = r == ny - 1 ? 0 : r + 1;
   const int oc = r * sx, om = rm * sx, op = rp * sx;
@@ -226,7 +226,7 @@ struct NoHook {
 // (TY + 2) x (TX + 2) densities).  (x0, y0): tile origin; st: the layout.
 // Periodic wrap.
 template <typename real, typename store_t, int TY, bool XP = false>
-__device__ __forceinline__ void load_tile(const store_t* __restrict__ fin, int nx, int ny, Strides st, int x0,
+__device__ __forceinline__ void load_tile(const store_t* fin, int nx, int ny, Strides st, int x0,
                                           int y0, real (&f)[kTileRows][9], real (*rs)[kTileX + 2]) {
   using Shape = TileShape<TY>;
   using M = NodeMap<TY, XP>;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void load_tile(const store_t* __restrict__ fin, int n
 // before_sync() runs after all phase-1 loads are issued and before the block
 // barrier (the batched kernel stores its lattice coefficients there).
 template <typename V, typename store_t, int TY, typename Hook = NoHook, bool XP = false>
-__device__ __forceinline__ void step_tile(const store_t* __restrict__ fin, store_t* __restrict__ fout, int nx,
+__device__ __forceinline__ void step_tile(const store_t* fin, store_t* __restrict__ fout, int nx,
                                           int ny, Strides st, const VCoef<V>& c, const LatCoef<V>& l, int x0, int y0,
                                           typename LaneType<V>::type (*rs)[kTileX + 2],
                                           const Hook& before_sync = Hook(), Rounding rnd = Rounding{0u, 0}) {
@@ -296,7 +296,7 @@ constexpr int fused_min_blocks() {
 }
 template <typename V, typename store_t>
 __global__ void __launch_bounds__(TileShape<kFusedRows>::threads, fused_min_blocks<V, store_t>())
-    k_step_fused(const store_t* __restrict__ fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
+    k_step_fused(const store_t* fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
                  VCoef<V> c, Rounding rnd) {
   follow_predecessor();
   rnd = resolve(rnd);
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(TileShape<kFusedRows>::threads, fused_min_bloc
 
 // Two-pass variant, pass 1: density plane rho_dev(x) = sum_i fbar_i(x - e_i).
 template <typename real, typename store_t>
-__global__ void k_density(const store_t* __restrict__ fin, real* __restrict__ rho, int nx, int ny, Strides st) {
+__global__ void k_density(const store_t* fin, real* __restrict__ rho, int nx, int ny, Strides st) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= nx || y >= ny) return;
   real f[9];
@@ -318,7 +318,7 @@ __global__ void k_density(const store_t* __restrict__ fin, real* __restrict__ rh
 
 // Two-pass variant, pass 2: pull, force stencil from the density plane, collide.
 template <typename real, typename store_t>
-__global__ void k_collide_rho(const store_t* __restrict__ fin, store_t* __restrict__ fout,
+__global__ void k_collide_rho(const store_t* fin, store_t* __restrict__ fout,
                               const real* __restrict__ rho, int nx, int ny, Strides st, VCoef<real> c,
                               Rounding rnd) {
   rnd = resolve(rnd);

@@ -190,7 +190,7 @@ __device__ __forceinline__ void cp_async_wait_all_but_one() { asm volatile("cp.a
 // All threads: the window of the (wrapping) tile at (x0, y0) of a lattice with
 // populations at fin (16-byte aligned; layout st) into win.  Plane i's window row r
 // holds lattice row y0 - 1 - e_iy + r, window column c lattice column x0 - 4 + c.
-__device__ __forceinline__ void issue_window_async(float* win, const float* __restrict__ fin, int nx, int ny,
+__device__ __forceinline__ void issue_window_async(float* win, const float* fin, int nx, int ny,
                                                    Strides st, int x0, int y0) {
   const int j = threadIdx.x;
   if (j < kAsyncThreads) {
@@ -311,7 +311,7 @@ __host__ __device__ __forceinline__ int tile_kind(int x0, int y0, int nx, int ny
 // S: storage type (float, or __half with the stores rounded as rnd says).
 template <typename V, typename S, bool ASYNC_EDGES>
 __global__ void __launch_bounds__(kFusedThreads, kTmaMinBlocks)
-    k_step_tma(const __grid_constant__ CUtensorMap tin, const S* __restrict__ fin, S* __restrict__ fout, int nx,
+    k_step_tma(const __grid_constant__ CUtensorMap tin, const S* fin, S* __restrict__ fout, int nx,
                int ny, Strides st, VCoef<V> c, int* __restrict__ err, Rounding rnd) {
   static_assert(!ASYNC_EDGES || sizeof(S) == 4, "asynchronous edge windows exist for FP32 storage only");
   rnd = resolve(rnd);
@@ -413,7 +413,7 @@ struct Win2 {
 
 template <typename V, typename S>
 __global__ void __launch_bounds__(kFusedThreads, kTmaMinBlocks)
-    k_step_tma_dyn(const __grid_constant__ CUtensorMap tin, const S* __restrict__ fin, S* __restrict__ fout, int nx,
+    k_step_tma_dyn(const __grid_constant__ CUtensorMap tin, const S* fin, S* __restrict__ fout, int nx,
                    int ny, Strides st, VCoef<V> c, int* __restrict__ err, Rounding rnd, unsigned* __restrict__ queue) {
   using real = float;
   follow_predecessor_only();
