@@ -16,6 +16,7 @@ struct ResPlan {
   int threads;       // of a block
   unsigned smem;     // dynamic shared memory of a block
   size_t words;      // 16-byte words of one parity of the exchange buffer, all tiles
+  int steps;         // at most, of one launch
 };
 }  // namespace lbm
 

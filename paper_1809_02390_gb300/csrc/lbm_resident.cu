@@ -29,6 +29,16 @@ size_t res_smem(int precision, int wmax, int hmax, int pitch) {
   return size_t(res_table_bytes(wmax, hmax, precision == LB_FP64 ? 1 : 2)) + plane * (real + 18 * store);
 }
 
+// Steps of one launch (even, so that a full chunk ends where it started): about 5 ms, so that
+// other work on the GPU gets its turn, by the plan's cost and some 3000 cycles a step of what
+// it leaves out (FP32 256^2 4,300 cycles a step, estimated 4,200; FP64 64^2 15,600 / 18,100;
+// FP64 410^2 at 9 rounds of warps 138,000, 72 steps: a fixed number of 4096 held the GPU for
+// 9 ms, 31 ms and some 0.3 s).
+int res_chunk(double cost) {
+  const int n = int(1e7 / (cost + 3000.0)) / 2 * 2;
+  return n < 16 ? 16 : n > 4096 ? 4096 : n;
+}
+
 }  // namespace
 
 // The cut with the smallest estimated step: a block's warps take the collision in
@@ -57,7 +67,7 @@ bool res_plan(int nx, int ny, int precision, ResPlan* out) {
       const int items = res_slots(w, h, lanes).total;
       const int warps = (items + 31) / 32;
       const double work = fp64 ? 15000.0 * ((warps + 3) / 4) : (130.0 * warps > 900.0 ? 130.0 * warps : 900.0);
-      const double cost = work + 4.0 * (w + h) + 0.01 * gx * gy;
+      const double cost = work + 4.0 * (w + h) + 0.01 * gx * gy;  // cycles
       if (found && cost >= best) continue;
       best = cost;
       found = true;
@@ -65,7 +75,7 @@ bool res_plan(int nx, int ny, int precision, ResPlan* out) {
       int threads = ((items + rounds - 1) / rounds + 31) / 32 * 32;
       if (threads < 128) threads = 128;
       *out = ResPlan{gx, gy, w, h, pitch, threads, unsigned(res_smem(precision, w, h, pitch)),
-                     size_t(gx) * gy * 6 * (w + h) * (fp64 ? 2 : 1)};
+                     size_t(gx) * gy * 6 * (w + h) * (fp64 ? 2 : 1), res_chunk(cost)};
     }
   return found;
 }
@@ -142,14 +152,12 @@ cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout,
 
 }  // namespace
 
-// Steps of one launch: a few milliseconds, so that other work on the GPU gets its turn.
-constexpr int64_t kResChunk = 4096;
-
 cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
   int64_t first = every;  // steps until the next recorded state
   while (nsteps > 0) {
     // Never a launch of one step: it could not write its result in place.
-    int64_t n = nsteps <= kResChunk ? nsteps : (nsteps == kResChunk + 1 ? kResChunk - 2 : kResChunk);
+    const int64_t chunk = h->res.steps;
+    const int64_t n = nsteps <= chunk ? nsteps : (nsteps == chunk + 1 ? chunk - 2 : chunk);
     const void* in = h->f[h->cur];
     void* out = h->f[n & 1 ? 1 - h->cur : h->cur];
     cudaError_t e;
