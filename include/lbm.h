@@ -393,6 +393,15 @@ enum lb_step_kind {
 };
 int lb_step_form(const lb_handle* h, int64_t nsteps);
 
+/* Resident runs of this handle (lb_step): -1 (the default) by rule, 0 never, 1 whenever the
+ * lattice fits and a call has steps enough.  Resident runs hold their SMs to the end, so
+ * lattices that step on streams of their own take turns once the GPU is full, where single
+ * launches share it; the rule therefore leaves resident runs while more streams of the device
+ * hold live handles of such lattices than runs of this one fit the GPU side by side (FP32
+ * 64^2 five, 256^2 two, 512^2 one).  Same bits either way.  LB_ENOTSUP for 1 where the lattice
+ * or its scratch buffer does not allow it, LB_EINVAL for other values. */
+int lb_set_resident(lb_handle* h, int mode);
+
 /* Measurement aid (no counterpart in the paper): one pass with the step's memory
  * traffic and none of its arithmetic, a copy of the state into the other buffer
  * reading and writing every population in place, tile by tile as the step (32 x 16

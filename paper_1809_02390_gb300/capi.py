@@ -59,6 +59,7 @@ SIGNATURES = [
     ("lb_step", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_step_record", ctypes.c_int, [_V, ctypes.c_int64, ctypes.c_int64, _V]),
     ("lb_step_form", ctypes.c_int, [_V, ctypes.c_int64]),
+    ("lb_set_resident", ctypes.c_int, [_V, ctypes.c_int]),
     ("lb_state", _V, [_V]),
     ("lb_steps_done", ctypes.c_int64, [_V]),
     ("lb_moments", ctypes.c_int, [_V, _V, _V, _V]),
@@ -194,6 +195,10 @@ def lb_step_form(h: int, nsteps: int) -> int:
     if form < 0:
         raise LBError(form, "lb_step_form: null handle or nsteps < 1")
     return form
+
+
+def lb_set_resident(h: int, mode: int) -> None:
+    check(lib().lb_set_resident(h, int(mode)), h)
 
 
 def lb_state(h: int) -> int:

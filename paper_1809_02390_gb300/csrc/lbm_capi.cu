@@ -210,9 +210,17 @@ int launch_form(const lb_handle* h) {
   return h->use_dyn ? LB_STEP_TENSOR_TICKETS : LB_STEP_TENSOR_WALK;
 }
 
-// Whether a call of nsteps steps runs resident (outside a capture).
+// Whether a call of nsteps steps runs resident (outside a capture): from `least` steps on,
+// while the streams that hold lattices which could are no more than the runs of this one that
+// fit the GPU side by side, or as lb_set_resident says.  A run beyond those waits for a whole
+// launch of another, while single launches share the GPU (us a step of k lattices on k streams,
+// resident / graphs of k_step_fused: FP32 64^2, 5 fit: k = 4 2.1 / 2.2, 6 4.0 / 2.3; 200 x 180, 3
+// fit: 3 2.8 / 3.3, 4 4.9 / 3.3; 256^2, 2 fit: 2 2.9 / 3.5, 3 5.4 / 3.3, 8 11.8 / 6.1; 512^2, 1 fits:
+// 1 3.9 / 4.6, 2 7.8 / 5.8; FP16 256^2: 2 3.5 / 3.7, 3 6.5 / 4.0; FP64 64^2: 4 15.0 / 16.1, 6 27.0 / 20.5;
+// 256^2: 1 28.6 / 30.3, 2 57.2 / 54.9).
 bool resident_call(const lb_handle* h, int64_t nsteps, int64_t least) {
-  return h->use_res && !h->forced_blocks && !h->forced_dispatch && nsteps >= least;
+  if (!h->use_res || h->forced_blocks || h->forced_dispatch || h->res_mode == 0 || nsteps < least) return false;
+  return h->res_mode == 1 || res_streams(h) <= h->res_fit;
 }
 
 template <typename V, typename real, typename store_t>
@@ -393,6 +401,7 @@ void release_wait_slot(lb_handle* h) {
 
 void destroy(lb_handle* h) {
   if (!h) return;
+  res_leave(h);
   release_wait_slot(h);
   for (int k = 0; k < 2; ++k) {
     if (h->graph[k]) cudaGraphExecDestroy(h->graph[k]);
@@ -642,6 +651,7 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
   h->c2 = make_vcoef<f2>(h->p, d);
   h->cd = make_vcoef<double>(h->p, d);
   h->wait_slot = -1;
+  h->res_dev = -1;
   h->graph_k = -1;
   rc = configure(h);
   if (rc != LB_OK) {
@@ -1040,6 +1050,15 @@ int lb_set_tile_dispatch(lb_handle* h, int dynamic) {
     return fail(h, LB_ENOTSUP, "dynamic dispatch needs the tensor-copy step and the scratch buffer");
   h->use_dyn = dynamic != 0;
   h->forced_dispatch = h->use_tma;
+  return LB_OK;
+}
+
+int lb_set_resident(lb_handle* h, int mode) {
+  if (!h) return fail(nullptr, LB_EINVAL, "null handle");
+  if (mode < -1 || mode > 1) return fail(h, LB_EINVAL, "mode must be -1, 0 or 1");
+  if (mode == 1 && !h->use_res)
+    return fail(h, LB_ENOTSUP, "the lattice does not fit a resident run, or its scratch has no exchange words");
+  h->res_mode = mode;
   return LB_OK;
 }
 

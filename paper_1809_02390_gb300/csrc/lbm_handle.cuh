@@ -56,6 +56,9 @@ struct lb_handle {
   bool forced_dispatch;   // lb_set_tile_dispatch asked for a tensor-copy form
   bool forced_blocks;     // lb_set_step_blocks fixed its grid
   lbm::ResPlan res;
+  int res_mode;           // lb_set_resident: -1 by rule, 0 never, 1 always
+  int res_fit;            // resident runs of this lattice that fit the GPU side by side
+  int res_dev;            // device of the handle's entry among the live resident handles (-1: none)
   void* res_mail;         // exchange words (end of the scratch buffer)
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
   bool overlap;           // the steps' launches may overlap their predecessor's end (lbm_launch.cuh)
@@ -86,6 +89,10 @@ size_t res_mail_bytes(int nx, int ny);
 // Decides whether the handle can run resident with the exchange buffer `mail` (device
 // memory of res_mail_bytes, 16-byte aligned, or null; its contents do not matter).
 cudaError_t res_configure(lb_handle* h, void* mail);
+// Takes the handle out of the live ones (lb_free).
+void res_leave(lb_handle* h);
+// Streams of the handle's device that live handles which can run resident are bound to.
+int res_streams(const lb_handle* h);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
 // null): device memory that receives the states after every `every` (< 2^31) steps.
 cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every);

@@ -3,6 +3,10 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+#include <mutex>
+#include <vector>
+
 #include "lbm_resident.cuh"
 #include "lbm_handle.cuh"
 
@@ -96,8 +100,53 @@ size_t res_mail_bytes(int nx, int ny) {
   return 2 * words * sizeof(uint4);
 }
 
+namespace {
+// Live handles that can run resident, by device and stream (an entry goes with its last
+// handle), and the number of streams per device, which every step call reads.
+struct Live {
+  int dev;
+  cudaStream_t stream;
+  int handles;
+};
+constexpr int kDevices = 64;
+std::mutex g_live_mu;
+std::vector<Live> g_live;
+std::atomic<int> g_live_streams[kDevices];
+
+void res_enter(lb_handle* h, int dev) {
+  std::lock_guard<std::mutex> lock(g_live_mu);
+  h->res_dev = dev;
+  for (Live& l : g_live)
+    if (l.dev == dev && l.stream == h->stream) {
+      ++l.handles;
+      return;
+    }
+  g_live.push_back(Live{dev, h->stream, 1});
+  ++g_live_streams[dev % kDevices];
+}
+}  // namespace
+
+void res_leave(lb_handle* h) {
+  if (!h || h->res_dev < 0) return;
+  std::lock_guard<std::mutex> lock(g_live_mu);
+  for (size_t k = 0; k < g_live.size(); ++k)
+    if (g_live[k].dev == h->res_dev && g_live[k].stream == h->stream) {
+      if (--g_live[k].handles == 0) {
+        g_live.erase(g_live.begin() + k);
+        --g_live_streams[h->res_dev % kDevices];
+      }
+      break;
+    }
+  h->res_dev = -1;
+}
+
+int res_streams(const lb_handle* h) {
+  return h->res_dev < 0 ? 0 : g_live_streams[h->res_dev % kDevices].load(std::memory_order_relaxed);
+}
+
 cudaError_t res_configure(lb_handle* h, void* mail) {
   h->use_res = false;
+  h->res_mode = -1;
   ResPlan p;
   // FP32 and FP16 up to kResNodes: above, a tile's pitch no longer avoids bank conflicts
   // and a step is no faster than a launch of k_step_fused (us: FP32 576^2 4.9 against 5.3,
@@ -116,7 +165,9 @@ cudaError_t res_configure(lb_handle* h, void* mail) {
   if (!coop || per_sm < 1 || sms < p.gx * p.gy) return cudaSuccess;
   h->res = p;
   h->res_mail = mail;
+  h->res_fit = per_sm * sms / (p.gx * p.gy);
   h->use_res = true;
+  res_enter(h, dev);
   return cudaSuccess;
 }
 
