@@ -402,6 +402,12 @@ int lb_step_form(const lb_handle* h, int64_t nsteps);
  * or its scratch buffer does not allow it, LB_EINVAL for other values. */
 int lb_set_resident(lb_handle* h, int mode);
 
+/* Test of a refused resident launch, on the host: after `launches` >= 0 more of them the next
+ * one is taken for refused by the device (as in a context with fewer SMs) and not made.  The
+ * call that meets it goes on by single launches, with the same bits, and the handle runs
+ * resident no more.  LB_ENOTSUP for a handle that does not. */
+int lb_resident_selftest(lb_handle* h, int64_t launches);
+
 /* Measurement aid (no counterpart in the paper): one pass with the step's memory
  * traffic and none of its arithmetic, a copy of the state into the other buffer
  * reading and writing every population in place, tile by tile as the step (32 x 16

@@ -60,6 +60,7 @@ SIGNATURES = [
     ("lb_step_record", ctypes.c_int, [_V, ctypes.c_int64, ctypes.c_int64, _V]),
     ("lb_step_form", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_set_resident", ctypes.c_int, [_V, ctypes.c_int]),
+    ("lb_resident_selftest", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_state", _V, [_V]),
     ("lb_steps_done", ctypes.c_int64, [_V]),
     ("lb_moments", ctypes.c_int, [_V, _V, _V, _V]),
@@ -199,6 +200,10 @@ def lb_step_form(h: int, nsteps: int) -> int:
 
 def lb_set_resident(h: int, mode: int) -> None:
     check(lib().lb_set_resident(h, int(mode)), h)
+
+
+def lb_resident_selftest(h: int, launches: int) -> None:
+    check(lib().lb_resident_selftest(h, int(launches)), h)
 
 
 def lb_state(h: int) -> int:

@@ -808,8 +808,9 @@ int lb_step(lb_handle* h, int64_t nsteps) {
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
   if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_steps(h))) {
-    LB_CUDA(h, res_run(h, nsteps, nullptr, 1));
-    return LB_OK;
+    int64_t done = 0;
+    LB_CUDA(h, res_run(h, nsteps, nullptr, 1, &done));
+    nsteps -= done;  // none left, unless the device refused a launch
   }
   if (nsteps >= kStepGraph && !h->graph_off && capture == cudaStreamCaptureStatusNone) {
     if (!ensure_step_graph(h)) {
@@ -856,8 +857,21 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
   h->overlap = capture == cudaStreamCaptureStatusNone;
   if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_record(h)) &&
       record_by_elements(h->p, reinterpret_cast<uintptr_t>(at))) {
-    LB_CUDA(h, res_run(h, nsteps, states, every));
-    return LB_OK;
+    int64_t done = 0;
+    LB_CUDA(h, res_run(h, nsteps, states, every, &done));
+    if (done == nsteps) return LB_OK;
+    // A launch was refused: to the next state by single launches, and on from there.
+    at += size_t(done / every) * bytes;
+    nsteps -= done;
+    if (done % every) {
+      const int64_t rest = every - done % every;
+      if (nsteps < rest) return lb_step(h, nsteps);
+      const int rc = lb_step(h, rest);
+      if (rc != LB_OK) return rc;
+      LB_CUDA(h, cudaMemcpyAsync(at, h->f[h->cur], bytes, cudaMemcpyDeviceToDevice, h->stream));
+      at += bytes;
+      nsteps -= rest;
+    }
   }
   if (every == 1 && record_in_place(h->p, reinterpret_cast<uintptr_t>(at), bytes, h->use_tma)) {
     // Every state is wanted: step from each straight into the next (the handle's buffers
@@ -1059,6 +1073,14 @@ int lb_set_resident(lb_handle* h, int mode) {
   if (mode == 1 && !h->use_res)
     return fail(h, LB_ENOTSUP, "the lattice does not fit a resident run, or its scratch has no exchange words");
   h->res_mode = mode;
+  return LB_OK;
+}
+
+int lb_resident_selftest(lb_handle* h, int64_t launches) {
+  if (!h) return fail(nullptr, LB_EINVAL, "null handle");
+  if (launches < 0) return fail(h, LB_EINVAL, "launches must be >= 0");
+  if (!h->use_res) return fail(h, LB_ENOTSUP, "the lattice does not run resident");
+  h->res_refuse = launches;
   return LB_OK;
 }
 

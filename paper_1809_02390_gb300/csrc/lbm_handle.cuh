@@ -58,6 +58,7 @@ struct lb_handle {
   lbm::ResPlan res;
   int res_mode;           // lb_set_resident: -1 by rule, 0 never, 1 always
   int res_fit;            // resident runs of this lattice that fit the GPU side by side
+  int64_t res_refuse;     // lb_resident_selftest: launches until one is taken for refused (-1: none)
   int res_dev;            // device of the handle's entry among the live resident handles (-1: none)
   void* res_mail;         // exchange words (end of the scratch buffer)
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
@@ -95,7 +96,9 @@ void res_leave(lb_handle* h);
 int res_streams(const lb_handle* h);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
 // null): device memory that receives the states after every `every` (< 2^31) steps.
-cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every);
+// *done: the steps taken; fewer than nsteps if the device refused a launch, in which case the
+// handle no longer runs resident.
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every, int64_t* done);
 // Device address of lb_reduce_static's static scratch on the current device
 // (looked up once per device, which commits the array there; lbm_static.cu).
 int static_scratch_address(lb_handle* h, void** out);

@@ -147,6 +147,7 @@ int res_streams(const lb_handle* h) {
 cudaError_t res_configure(lb_handle* h, void* mail) {
   h->use_res = false;
   h->res_mode = -1;
+  h->res_refuse = -1;
   ResPlan p;
   // FP32 and FP16 up to kResNodes: above, a tile's pitch no longer avoids bank conflicts
   // and a step is no faster than a launch of k_step_fused (us: FP32 576^2 4.9 against 5.3,
@@ -203,19 +204,36 @@ cudaError_t launch(lb_handle* h, const VCoef<V>& c, const void* fin, void* fout,
 
 }  // namespace
 
-cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
+// Launches that the device refuses for what else limits the stream (a green context with
+// fewer SMs than the device, a debugger's or a partition's limits): single launches still run.
+bool res_refused(cudaError_t e) {
+  return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported ||
+         e == cudaErrorInvalidConfiguration || e == cudaErrorNotPermitted;
+}
+
+cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every, int64_t* done) {
   int64_t first = every;  // steps until the next recorded state
-  while (nsteps > 0) {
+  *done = 0;
+  while (*done < nsteps) {
     // Never a launch of one step: it could not write its result in place.
-    const int64_t chunk = h->res.steps;
-    const int64_t n = nsteps <= chunk ? nsteps : (nsteps == chunk + 1 ? chunk - 2 : chunk);
+    const int64_t chunk = h->res.steps, left = nsteps - *done;
+    const int64_t n = left <= chunk ? left : (left == chunk + 1 ? chunk - 2 : chunk);
     const void* in = h->f[h->cur];
     void* out = h->f[n & 1 ? 1 - h->cur : h->cur];
     cudaError_t e;
-    switch (h->p.precision) {
-      case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, int(first), int(every), int(n)); break;
-      case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
-      default: e = launch<f2, __half>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
+    if (h->res_refuse >= 0 && h->res_refuse-- == 0)
+      e = cudaErrorCooperativeLaunchTooLarge;  // lb_resident_selftest
+    else
+      switch (h->p.precision) {
+        case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, int(first), int(every), int(n)); break;
+        case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
+        default: e = launch<f2, __half>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
+      }
+    if (res_refused(e)) {
+      cudaGetLastError();
+      h->use_res = false;
+      res_leave(h);
+      return cudaSuccess;
     }
     if (e != cudaSuccess) return e;
     if (rec) {
@@ -225,7 +243,7 @@ cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every) {
     }
     h->steps += n;
     if (n & 1) h->cur = 1 - h->cur;
-    nsteps -= n;
+    *done += n;
   }
   return cudaSuccess;
 }
