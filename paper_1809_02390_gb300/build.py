@@ -13,23 +13,25 @@ LIB = os.path.join(BUILD, "liblbm.so")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["lbm_capi.cu", "lbm_static.cu", "lbm_resident.cu", "lbm_adjoint.cu", "lbm_batch.cu", "lbm3d.cu", "lbm_thermo.cpp"]
-HEADERS = ["lbm_internal.h", "lbm_device.cuh", "lbm_kernels.cuh", "lbm_handle.cuh", "lbm_adjoint.cuh", "lbm_tma.cuh",
-           "lbm_fields.cuh", "lbm_resident.cuh", "lbm3d_step.cuh"]
-COMMON = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(HERE, "..", "include")]
+INCLUDE = os.path.join(HERE, "..", "include")
+COMMON = ["-O3", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE]
 
 
 def _sources() -> list[str]:
     return [s for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
 
 
+def dependencies() -> list[str]:
+    """The sources and every header beside them or in include/."""
+    headers = [os.path.join(d, f) for d in (CSRC, INCLUDE) for f in sorted(os.listdir(d)) if f.endswith((".h", ".cuh"))]
+    return [os.path.join(CSRC, s) for s in _sources()] + headers
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, s) for s in _sources()] + [os.path.join(CSRC, h) for h in HEADERS]
-    deps.append(os.path.join(HERE, "..", "include", "lbm.h"))
-    deps.append(os.path.join(HERE, "..", "include", "lbm3d.h"))
-    return any(os.path.exists(d) and os.path.getmtime(d) > t for d in deps)
+    return any(os.path.getmtime(d) > t for d in dependencies())
 
 
 def _compile(src: str, verbose: bool) -> str:
