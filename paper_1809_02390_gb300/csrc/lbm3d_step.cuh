@@ -138,7 +138,7 @@ struct CV3 {
   V nsp, nbq5;                   // -s_p, -5 bq / 3
   V sq6, om8;                    // s_q / 6, (1 - s_m) / 8
   V one, two, three, half, quarter, nquarter, eighth, n2, n3, n4, nhalf;
-  V third, nthird, sixth, n12, twelfth, i24, n2h, n5h, n10h, c1375, c1121;
+  V nthird, sixth, n12, i24, n2h, n5h, n10h, c1375, c1121;
 };
 
 // Post-collision populations of one node (two for V = f2) from the rest population f0,
