@@ -2,6 +2,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -237,7 +238,6 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
   }
   const int form = launch_form(h);
   if (form != LB_STEP_TWO_PASS) {
-    const dim3 grd((nx + kTileX - 1) / kTileX, (ny + kFusedRows - 1) / kFusedRows);
     if constexpr (sizeof(store_t) <= 4 && std::is_same<V, f2>::value) {
       if (form == LB_STEP_TENSOR_TICKETS) {
         launch_step_kernel(h->overlap, k_step_tma_dyn<V, store_t>, h->dyn_grid, kFusedThreads, Win2<store_t>::smem,
@@ -250,8 +250,11 @@ void launch_step(lb_handle* h, const VCoef<V>& cv, const VCoef<real>& c) {
         return;
       }
     }
-    launch_step_kernel(h->overlap, k_step_fused<V, store_t>, grd, TileShape<kFusedRows>::threads, 0, h->stream, fin,
-                       fout, nx, ny, h->st, cv, rnd);
+    // (Several launches for lattices of more than 524,280 rows, the limit of a grid in y.)
+    const int cols = (nx + kTileX - 1) / kTileX, rows = (ny + kFusedRows - 1) / kFusedRows;
+    for (int row0 = 0; row0 < rows; row0 += kFusedGridY)
+      launch_step_kernel(h->overlap, k_step_fused<V, store_t>, dim3(cols, std::min(rows - row0, kFusedGridY)),
+                         TileShape<kFusedRows>::threads, 0, h->stream, fin, fout, nx, ny, h->st, cv, rnd, row0);
   } else {
     real* rho = static_cast<real*>(h->scratch);
     const dim3 blk(32, 8), grd((nx + 31) / 32, (ny + 7) / 8);

@@ -284,6 +284,7 @@ __device__ __forceinline__ void step_tile(const store_t* fin, store_t* __restric
 // node.  FP32 and FP16: more, smaller blocks fill each other's load phases and the last
 // wave (FP32 1003 x 517 8.8 -> 7.9 us a step, 4095^2 261 -> 227, both at 80 registers).
 constexpr int kFusedRows = 8;
+constexpr int kFusedGridY = 65535;  // rows of tiles that one launch takes
 // Resident blocks per SM the register budget must allow.  FP32: 6 (80 registers).  With 64
 // registers the collision spills 124 bytes a thread, whose stores went through to L2 (twice
 // the write traffic of the step itself) and bounded it: 1003 x 517 10.5 us a step against
@@ -294,16 +295,17 @@ template <typename V, typename store_t>
 constexpr int fused_min_blocks() {
   return sizeof(typename LaneType<V>::type) == 8 ? 4 : sizeof(store_t) == 2 ? 7 : 6;
 }
+// row0: first row of tiles of this launch.
 template <typename V, typename store_t>
 __global__ void __launch_bounds__(TileShape<kFusedRows>::threads, fused_min_blocks<V, store_t>())
     k_step_fused(const store_t* fin, store_t* __restrict__ fout, int nx, int ny, Strides st,
-                 VCoef<V> c, Rounding rnd) {
+                 VCoef<V> c, Rounding rnd, int row0) {
   follow_predecessor();
   rnd = resolve(rnd);
   __shared__ __align__(16) typename LaneType<V>::type rs[kFusedRows + 2][kTileX + 2];
   constexpr bool XP = xpairs<store_t>() && Lanes<V>::n == 2;
   step_tile<V, store_t, kFusedRows, NoHook, XP>(fin, fout, nx, ny, st, c, lattice_part(c), blockIdx.x * kTileX,
-                                        blockIdx.y * kFusedRows, rs, NoHook(), rnd);
+                                        (blockIdx.y + row0) * kFusedRows, rs, NoHook(), rnd);
 }
 
 // Two-pass variant, pass 1: density plane rho_dev(x) = sum_i fbar_i(x - e_i).
