@@ -292,7 +292,8 @@ int lb_batch_run(lb_batch* b, int64_t nsteps);
  * blocks per SM; tensor copies: persistent grid of 1..max blocks per SM) for
  * trial_steps steps on the batch itself (advancing it) and keeps the fastest;
  * writes its time per step.  lb_batch_config reports blocks_per_sm = 0 for the
- * one-block-per-tile grid; lb_batch_uses_tma is 1 when the tensor-copy kernel is
+ * one-block-per-tile grid, the rows of a tile and the blocks of a launch (shape 1 without a
+ * persistent grid: two a tile, each for one 8-row half); lb_batch_uses_tma is 1 when the tensor-copy kernel is
  * the chosen shape. */
 int lb_batch_tune(lb_batch* b, int trial_steps, double* best_ms_per_step);
 int lb_batch_config(const lb_batch* b, int* tile_y, int* blocks_per_sm, int* grid);

@@ -437,6 +437,9 @@ int max_blocks(lb_batch* b, int shape, int* out) {
   return LB_OK;
 }
 
+// One block per 8-row half of a tile (shape 1 without a persistent grid).
+bool half_tiles(const lb_batch* b) { return b->shape == 1 && b->blocks_per_sm == 0; }
+
 void launch_one(lb_batch* b, int from) {
   const float* in = static_cast<const float*>(b->pool[from]);
   float* out = static_cast<float*>(b->pool[1 - from]);
@@ -463,7 +466,7 @@ void launch_one(lb_batch* b, int from) {
   } else if (s == 0)
     launch_shape<16, 4>(in, out, tiles, b->d_coef, total, b->blocks_per_sm, b->sms, b->common, b->stream, b->rows,
                         b->overlap);
-  else if (s == 1 && b->blocks_per_sm == 0)
+  else if (half_tiles(b))
     // One block per half tile: 8 rows, 6 blocks per SM at 80 registers.  Smaller blocks hide
     // each other's loads (48 lattices, 0.92 M nodes: 16.9 -> 14.4 us a step).
     launch_step_kernel(b->overlap, k_step_batch<float, 8, 6, false>, 2 * total, TileShape<8>::threads, 0, b->stream, in,
@@ -842,9 +845,10 @@ int lb_batch_tune(lb_batch* b, int trial_steps, double* best_ms_per_step) {
 
 int lb_batch_config(const lb_batch* b, int* tile_y, int* blocks_per_sm, int* grid) {
   if (!b) return LB_EINVAL;
+  const int parts = half_tiles(b) ? 2 : 1;  // blocks a tile
   if (tile_y) *tile_y = kShapeTY[b->shape];
   if (blocks_per_sm) *blocks_per_sm = b->blocks_per_sm;
-  if (grid) *grid = b->blocks_per_sm > 0 ? b->blocks_per_sm * b->sms : b->total_tiles[b->shape];
+  if (grid) *grid = b->blocks_per_sm > 0 ? b->blocks_per_sm * b->sms : b->total_tiles[b->shape] * parts;
   return LB_OK;
 }
 
