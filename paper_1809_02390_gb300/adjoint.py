@@ -132,7 +132,8 @@ def rollout(theta, f0, spec: RolloutSpec, nsteps: int, checkpoint_every: int | N
     (float64 tensor (Tr, G2, K_int)) and ``f0``."""
     if LBRollout.fn is None:
         LBRollout.fn = _make_function()
-    every = checkpoint_every or max(1, int(round(math.sqrt(nsteps))))
+    nsteps = int(nsteps)
+    every = int(checkpoint_every or max(1, round(math.sqrt(nsteps))))
     return LBRollout.fn.apply(theta, f0, spec, nsteps, every)
 
 

@@ -847,7 +847,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
 int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
   if (!h) return fail(nullptr, LB_EINVAL, "null handle");
   if (nsteps < 0) return fail(h, LB_EINVAL, "nsteps must be >= 0");
-  if (every < 1 || every > INT32_MAX) return fail(h, LB_EINVAL, "every must be in [1, 2^31)");
+  if (every < 1) return fail(h, LB_EINVAL, "every must be >= 1");
   if (nsteps < every) return lb_step(h, nsteps);
   if (!states) return fail(h, LB_EINVAL, "null state buffer");
   const size_t bytes = lb_state_bytes(&h->p);

@@ -95,7 +95,7 @@ void res_leave(lb_handle* h);
 // Streams of the handle's device that live handles which can run resident are bound to.
 int res_streams(const lb_handle* h);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
-// null): device memory that receives the states after every `every` (< 2^31) steps.
+// null): device memory that receives the states after every `every` steps.
 // *done: the steps taken; fewer than nsteps if the device refused a launch, in which case the
 // handle no longer runs resident.
 cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every, int64_t* done);

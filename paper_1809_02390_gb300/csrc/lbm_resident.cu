@@ -211,6 +211,9 @@ bool res_refused(cudaError_t e) {
          e == cudaErrorInvalidConfiguration || e == cudaErrorNotPermitted;
 }
 
+// (A launch takes at most 4096 steps, so larger distances are all the same to it.)
+static int to_int(int64_t v) { return v > INT32_MAX ? INT32_MAX : int(v); }
+
 cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every, int64_t* done) {
   int64_t first = every;  // steps until the next recorded state
   *done = 0;
@@ -225,9 +228,9 @@ cudaError_t res_run(lb_handle* h, int64_t nsteps, void* rec, int64_t every, int6
       e = cudaErrorCooperativeLaunchTooLarge;  // lb_resident_selftest
     else
       switch (h->p.precision) {
-        case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, int(first), int(every), int(n)); break;
-        case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
-        default: e = launch<f2, __half>(h, h->c2, in, out, rec, int(first), int(every), int(n)); break;
+        case LB_FP64: e = launch<double, double>(h, h->cd, in, out, rec, to_int(first), to_int(every), int(n)); break;
+        case LB_FP32: e = launch<f2, float>(h, h->c2, in, out, rec, to_int(first), to_int(every), int(n)); break;
+        default: e = launch<f2, __half>(h, h->c2, in, out, rec, to_int(first), to_int(every), int(n)); break;
       }
     if (res_refused(e)) {
       cudaGetLastError();
