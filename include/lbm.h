@@ -134,7 +134,7 @@ size_t lb_state_bytes(const lb_params* p);
 /* Bytes of device scratch memory: one density plane (two-pass variant, reductions),
  * the reduction workspace, 256 bytes of tile tickets (fused tensor-copy step) and, for
  * lattices that fit the SMs' shared memory, the exchange words of the resident run
- * (lb_step; at most 8 MB).  A buffer without the last part is accepted too: lb_step
+ * (lb_step; to 4 MB for squares, at most 18 MB for strips of three rows).  A buffer without the last part is accepted too: lb_step
  * then launches step by step. */
 size_t lb_scratch_bytes(const lb_params* p);
 
@@ -158,8 +158,8 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
             size_t scratch_bytes, const double* rho0, int rho0_on_device, void* stream);
 
 /* Advances nsteps >= 0 time steps (Eq. 13 + supplement Eq. 2) on the stream.
- * Asynchronous.  A small fused lattice (FP64 to about 485^2, FP32 and FP16 to 340,000
- * nodes) takes calls of several steps (at least 4, FP32 and FP16 12) in one cooperative
+ * Asynchronous.  A small fused lattice (FP64 to 410^2, FP32 and FP16 to 340,000 nodes,
+ * lb_step_form tells) takes calls of several steps (at least 4, FP32 and FP16 12) in one cooperative
  * launch that keeps it in the SMs' shared memory (same bits; waits between its blocks are
  * bounded at 10 s and reported by lb_status), unless lb_set_step_blocks or
  * lb_set_tile_dispatch asked for a tensor-copy form (lb_step_form tells which form serves a call).  Else runs of 64 steps replay a CUDA graph that the handle captures on
