@@ -269,6 +269,9 @@ CV3<V> make_cv3(const lb_params& p, const lb_derived& d) {
   c.cA = m(cA);
   c.G2s = m(d.G2 / 12.0);
   c.gq = m(d.G2 / 1728.0);
+  c.lam_RT3_lo = Val<V>::low(3.0 * d.lam * RT);
+  c.cA_lo = Val<V>::low(cA);
+  c.G2s_lo = Val<V>::low(d.G2 / 12.0);
   c.se = m(d.s_e);
   c.kse = m(d.k * d.s_eps * om_e / 19.0);
   c.hq = m(d.h * d.s_q * om_e * 5.0 / 57.0);

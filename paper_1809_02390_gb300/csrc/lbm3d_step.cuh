@@ -104,6 +104,7 @@ struct Val<f2> {
     return fmav(r, fmav(-x, r, one), r);
   }
   static f2 make(double v) { return f2{make_float2(float(v), float(v))}; }
+  static f2 low(double v) { return make(v - double(float(v))); }  // what make leaves of v
 };
 template <>
 struct Val<r64> {
@@ -113,6 +114,7 @@ struct Val<r64> {
   __device__ static double get(r64 v, int) { return v.v; }
   __device__ static r64 rcp(r64 x) { return r64{lbm::rcp_fp64(x.v)}; }
   static r64 make(double v) { return r64{v}; }
+  static r64 low(double) { return r64{0.0}; }
 };
 template <typename T>
 struct ValOf;
@@ -132,6 +134,7 @@ struct CV3 {
   V rho_ref, nbq;                // rho_ref; -b (vdW) or -b / 4 (Carnahan-Starling)
   V lam_RT3, cA;                 // 3 lam R T, 3 G2 / 2 - 3 lam a
   V G2s, gq;                     // G2 / 12, G2 / 1728
+  V lam_RT3_lo, cA_lo, G2s_lo;   // FP32: what the rounded constants leave
   V se, kse, hq;                 // s_e, k s_eps om_e / 19, h s_q om_e 5 / 57 (om_e = s_e / 2 - 1)
   V ceta, seps_a;                // -(beta_2 + 11 / 2), 2 s_eps / 21
   V sp3, spi3, bq2, bq23, nbq23;  // s_p / 3, s_pi / 3, 10 bq / 3, 10 bq / 9, its negative (bq = b s_q om_p)
@@ -169,23 +172,40 @@ __device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9],
   // EOS: p_LBE = p_EOS + G^2 rho^2 / 2 (Eq. 18), eta = 3 p_LBE - rho (Eq. 9).
   const V rho = delta + c.rho_ref;
   V ir, p3;  // 1 / rho, 3 p_LBE
+  // 3 p_LBE / rho = lam_RT3 z + cA rho, z the EOS's factor.  The two terms nearly cancel, and
+  // the force must cancel the G^2 part of cA exactly in a flat interface, so in FP32 the
+  // rounding of the three constants is the largest error of the step (two-phase 24^3 lattices,
+  // 135 steps at T_r 0.857: 4.6e-7 to 6.8e-7 off 64 bits, 1.6e-7 to 2.0e-7 with the constants in
+  // two floats; collide3_moments 3.9e-7 to 5.5e-7).
+  constexpr bool kTwoFloats = Val<V>::lanes == 2;
+  auto slope = [&](V z) { return fmav(c.cA, rho, fmav(c.lam_RT3, z, fmav(c.lam_RT3_lo, z, c.cA_lo * rho))); };
   if (c.eos == LB_EOS_VDW) {
     const V om = fmav(c.nbq, rho, c.one);
     const V r = Val<V>::rcp(rho * om);
     ir = r * om;
-    p3 = rho * fmav(c.cA, rho, c.lam_RT3 * (r * rho));
+    if constexpr (kTwoFloats)
+      p3 = rho * slope(r * rho);
+    else
+      p3 = rho * fmav(c.cA, rho, c.lam_RT3 * (r * rho));
   } else {
     const V om = fmav(c.nbq, rho, c.one), t = c.one - om;
     const V r = Val<V>::rcp(rho * om);
     const V io = r * rho;
     ir = r * om;
     const V z = fmav(t * t, om, c.one + t) * (io * io * io);  // (1 + t + t^2 - t^3) / (1 - t)^3
-    p3 = rho * fmav(c.lam_RT3, z, c.cA * rho);
+    if constexpr (kTwoFloats)
+      p3 = rho * slope(z);
+    else
+      p3 = rho * fmav(c.lam_RT3, z, c.cA * rho);
   }
   const V eta = p3 - rho;
 
   // Force (Eq. 12), velocity (Eq. 5) and their products.
-  const V G2r = c.G2s * rho;
+  V G2r;
+  if constexpr (kTwoFloats)
+    G2r = fmav(c.G2s, rho, c.G2s_lo * rho);
+  else
+    G2r = c.G2s * rho;
   const V Fx = G2r * sx, Fy = G2r * sy, Fz = G2r * sz;
   const V Jx = fmav(c.half, Fx, jx), Jy = fmav(c.half, Fy, jy), Jz = fmav(c.half, Fz, jz);
   const V ux = Jx * ir, uy = Jy * ir, uz = Jz * ir;
@@ -266,7 +286,7 @@ __device__ __forceinline__ void collide3(const CV3<V>& c, V f0, const V (&s)[9],
   // 2e-10 and 6e-7); summing the 18 first and taking them off at once leaves 1e-10 a step.
   // FP64 has no such drift to speak of (1e-18 a step) and its pipe no room for 14
   // instructions more.
-  if constexpr (Val<V>::lanes == 2) {
+  if constexpr (kTwoFloats) {
     V t = delta;
 #pragma unroll
     for (int P = 0; P < 9; ++P) t = t - (o[2 * P + 1] + o[2 * P + 2]);
