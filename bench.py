@@ -44,14 +44,14 @@ KERNEL_SOURCES = ["paper_1809_02390_gb300/csrc/lbm_kernels.cuh", "paper_1809_023
 # layout and the hash of its sources (a changed kernel has no figure until recaptured).
 NCU_TRAFFIC = {
     # 2048^2 capture (profiles/k_step_tma_dyn_fp32_rows_2048_full.md) scaled x4 to 4096^2.
-    ("k_step_tma_dyn<f2>", "rows", "e5b676ce7b6e4e02"): 1019841536,
+    ("k_step_tma_dyn<f2>", "rows", "0244e3f6f58a4934"): 1022717952,
 }
 # The same for the D3Q19 step, keyed by the hash of its step code (csrc/lbm3d_step.cuh):
 # the 192^3 capture (profiles/k_d3_step_fp32_192cubed_full.md) scaled by the node
 # count to 256^3.
 KERNEL_SOURCES_D3Q19 = ["paper_1809_02390_gb300/csrc/lbm3d_step.cuh"]
 NCU_TRAFFIC_D3Q19 = {
-    ("k_d3_step<float, true>", "79edb1409287a483"): 2664552978,
+    ("k_d3_step<float, true>", "d5a1a09f23e141d4"): 2731334770,
 }
 
 
@@ -590,10 +590,11 @@ def run_ours(args):
     lat = Lattice(rho0, precision=main_prec, variant=main_var, Tr=TR, layout=args.layout)
     if args.dispatch == "static" and capi.lb_tile_dispatch(lat.h):
         capi.lb_set_tile_dispatch(lat.h, False)
-    tensor = capi.lb_uses_tma(lat.h) and (args.dispatch == "static" or
-                                          2 * lat.f_a.numel() * lat.f_a.element_size() > 100 << 20)
-    kernel = ("k_step_tma_dyn<f2>" if capi.lb_tile_dispatch(lat.h) else "k_step_tma<f2>") if tensor \
-        else ("k_step_fused<f2,float>" if main_var == "fused" else "k_density + k_collide_rho")
+    kernel = {capi.LB_STEP_TWO_PASS: "k_density + k_collide_rho", capi.LB_STEP_PLAIN: "k_step_fused",
+              capi.LB_STEP_TENSOR_WALK: "k_step_tma", capi.LB_STEP_TENSOR_TICKETS: "k_step_tma_dyn",
+              capi.LB_STEP_RESIDENT: "k_resident"}[capi.lb_step_form(lat.h, args.steps)]
+    if kernel.startswith("k_step") or kernel == "k_resident":
+        kernel += "<double>" if main_prec == "fp64" else "<f2>"
     lat.step(args.warmup)
     barrier(world)
     with ClockSampler(torch.cuda.current_device()) as clk:
@@ -682,7 +683,7 @@ def run_ours(args):
         lt.step(3)
         m = time_steps(lt, k, torch) / k
         gbs = BYTES_PER_LU_D3Q19[prec] * n3 ** 3 / (m * 1e-3) / 1e9
-        kern = "k_d3_step<%s>" % ("float, true" if prec == "fp32" else "double, false")
+        kern = "k_d3_step<%s>" % ("float, true" if prec == "fp32" else "double, true")
         sha3 = kernel_source_hash(KERNEL_SOURCES_D3Q19)
         tr3 = NCU_TRAFFIC_D3Q19.get((kern, sha3))
         variants["d3q19_%s_256cubed" % prec] = {
@@ -709,7 +710,7 @@ def run_ours(args):
     variants["d3q19_fp32_512cubed"] = {
         "MLUPS": round(n5 ** 3 / (m * 1e-3) / 1e6, 1), "ms_per_step": round(m, 4), "steps": k5,
         "algorithmic_GBps": round(gbs, 1), "frac_of_measured_hbm": round(gbs / pk["hbm_gbs"], 4),
-        "kernel": "k_d3_step<float, true, long long> (64-bit plane offsets)"}
+        "kernel": "k_d3_step<float, true> (64-bit plane offsets)"}
     lt.close()
     del lt
     torch.cuda.empty_cache()
