@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(kFusedThreads, MINB)
                          const TileRec* __restrict__ tiles, const LatCoef<f2>* __restrict__ coef,
                          const CUtensorMap* __restrict__ maps, int total_tiles, VCoef<f2> common,
                          int* __restrict__ err, unsigned* __restrict__ queue, int rows) {
-  follow_predecessor_only();
+  follow_predecessor();
   extern __shared__ __align__(128) unsigned char dyn[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
   __shared__ float rs[2][kTileY + 2][kTileX + 2];

@@ -3,15 +3,20 @@
 // A step reads what the step before it wrote, so its blocks wait for all of the
 // predecessor; but the launch itself (block scheduling, parameters, the first
 // instructions) need not.  Such a kernel begins with follow_predecessor() and is
-// launched by launch_step_kernel(): the blocks come up while the predecessor's last
-// ones finish and wait there until it is complete and its writes are visible.
+// launched by launch_step_kernel(): its blocks come up as the predecessor's blocks exit
+// and wait there until all of it is complete and its writes are visible.
 //
-// Measured, before -> after (us a step): a step of the adjoint at 256^2 FP32 6.3 -> 5.1;
-// D2Q9 FP32 1003 x 517 11.5 -> 11.2; rows layout FP32, 20 launches, 1024^2 18.7 -> 17.1,
-// 2048^2 54.5 -> 52.5, 4096^2 192.6 -> 190.5 (by graph 16.6 -> 16.4, 51.6 -> 51.5, 189.5 ->
-// 189.7; these three before follow_predecessor_only); D3Q19 FP32 64^3 14.4 -> 14.2, 256^3 469 -> 458; 48 lattices of a batch
-// 76.6 -> 75.6.  It costs nothing anywhere that was tried, so every step kernel is
-// launched so, except into a caller's own capture.
+// Measured, ordinary launch -> this (us a step): adjoint FP32 256^2 6.9 -> 5.0, 400^2 11.0 ->
+// 8.6; D2Q9 by graph FP32 256^2 2.61 -> 2.37, 1003 x 517 7.95 -> 7.74, FP16 450^2 4.80 -> 4.45,
+// FP64 256^2 30.7 -> 30.4, one launch a call FP32 512^2 6.3 -> 4.9; FP32 4096^2 187 -> 184.5; D3Q19
+// FP32 24 x 72 x 32 5.55 -> 5.3, 64^3 14.35 -> 14.07, 160^3 133.8 -> 133.4.  Nowhere that was
+// tried slower, so every step kernel is launched so, except into a caller's own capture.
+//
+// Measured and not kept: griddepcontrol.launch_dependents right after the wait, so that the
+// successor comes up while its predecessor runs.  Its blocks then take places next to the
+// running ones, several to an SM, and keep them, so the next step runs with its blocks
+// heaped: FP64 301 x 299 45.2 -> 59.2, adjoint 400^2 8.6 -> 9.8, D3Q19 48 x 32 x 32 5.35 -> 6.24
+// (slower than ordinary launches), 160^3 133.4 -> 140.4; at best 1% faster (52 x 50 x 219).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -22,17 +27,8 @@ namespace lbm {
 
 // All threads, before the first access to global memory.  Every block of a kernel that
 // is launched with launch_step_kernel waits here, whatever it does later, so that
-// "complete" includes all earlier steps.  The successor's blocks may come up as soon as
-// every block of this kernel has passed here.  (Nothing to wait for in an ordinary launch.)
-__device__ __forceinline__ void follow_predecessor() {
-  asm volatile("griddepcontrol.wait;\n griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// The same without the early start of the successor, whose blocks then come up as this
-// kernel's exit: for persistent kernels, where they would hold the SMs' free slots while
-// tiles are left (20 steps, against an ordinary launch and an early start: FP32 4096^2 3738,
-// 3704 -> 3689 us; FP16 4096 x 2048 2009, 1972 -> 1962).
-__device__ __forceinline__ void follow_predecessor_only() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// "complete" includes all earlier steps.  (Nothing to wait for in an ordinary launch.)
+__device__ __forceinline__ void follow_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // overlap = false: an ordinary launch (a caller's stream capture records plain edges).
 template <typename... P, typename... A>

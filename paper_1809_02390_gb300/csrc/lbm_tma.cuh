@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kFusedThreads, kTmaMinBlocks)
     k_step_tma_dyn(const __grid_constant__ CUtensorMap tin, const S* fin, S* __restrict__ fout, int nx,
                    int ny, Strides st, VCoef<V> c, int* __restrict__ err, Rounding rnd, unsigned* __restrict__ queue) {
   using real = float;
-  follow_predecessor_only();
+  follow_predecessor();
   rnd = resolve(rnd);
   static_assert(Win2<S>::buffer % 128 == 0, "window buffers start on 128-byte boundaries");
   extern __shared__ __align__(128) unsigned char dyn[];
