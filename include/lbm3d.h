@@ -98,6 +98,16 @@ int lb_d3_moments(lb_d3_handle* h, void* rho, void* ux, void* uy, void* uz);
  * that lb_d3_init allocates. */
 int lb_d3_reduce(lb_d3_handle* h, double out[8]);
 
+/* The form of the step.  WINDOWS: every plane's populations arrive in shared memory by
+ * asynchronous copies; PULLS (FP32): each thread loads its node's.  FP64 lattices take
+ * windows; FP32 ones the form that an estimate from the sides calls faster (windows need
+ * nx >= 40 and a multiple of 4, and buffers on 16 bytes).  FP32 rounds differently in the two.
+ * lb_d3_set_form fixes it (LB_D3_AUTO: by rule again; LB_ENOTSUP where the lattice does not
+ * allow the form); steps that are enqueued already keep theirs.  For tuning and tests. */
+enum lb_d3_step_form { LB_D3_AUTO = -1, LB_D3_PULLS = 0, LB_D3_WINDOWS = 1 };
+int lb_d3_form(const lb_d3_handle* h);
+int lb_d3_set_form(lb_d3_handle* h, int form);
+
 /* Synchronous health check: LB_ETIMEOUT if a bounded wait of the step's tensor copies
  * gave up since the last call (the flag is cleared), else LB_OK. */
 int lb_d3_status(lb_d3_handle* h);

@@ -114,6 +114,8 @@ SIGNATURES = [
     ("lb_d3_step", ctypes.c_int, [_V, ctypes.c_int64]),
     ("lb_d3_moments", ctypes.c_int, [_V, _V, _V, _V, _V]),
     ("lb_d3_reduce", ctypes.c_int, [_V, _D]),
+    ("lb_d3_form", ctypes.c_int, [_V]),
+    ("lb_d3_set_form", ctypes.c_int, [_V, ctypes.c_int]),
     ("lb_d3_status", ctypes.c_int, [_V]),
     ("lb_d3_state", _V, [_V]),
     ("lb_d3_get_state", ctypes.c_int, [_V, _V]),
@@ -185,6 +187,18 @@ def lb_step(h: int, nsteps: int) -> None:
 
 def lb_step_record(h: int, nsteps: int, every: int, states: int) -> None:
     check(lib().lb_step_record(h, int(nsteps), int(every), states), h)
+
+
+# Forms of the D3Q19 step (enum lb_d3_step_form).
+LB_D3_AUTO, LB_D3_PULLS, LB_D3_WINDOWS = -1, 0, 1
+
+
+def lb_d3_form(h: int) -> int:
+    return lib().lb_d3_form(h)
+
+
+def lb_d3_set_form(h: int, form: int) -> None:
+    check_d3(lib().lb_d3_set_form(h, int(form)), h)
 
 
 # Forms of a step call (enum lb_step_kind).

@@ -158,6 +158,8 @@ struct lb_d3_handle {
   C3<float> cpull;  // of k_d3_pull
   bool vec;         // rows of a multiple of 16 bytes (and both buffers aligned)
   bool windows;     // k_d3_step (else k_d3_pull)
+  bool can_window, can_pull, auto_windows;  // forms that the lattice allows, and the one by rule
+  int sms;
   bool have_maps;   // tensor maps of both buffers
   CUtensorMap maps[2];
   int* wait_error;  // device word set by a bounded wait that gave up (behind `part`)
@@ -315,6 +317,9 @@ CV3<V> make_cv3(const lb_params& p, const lb_derived& d) {
 // rounds of the full chunks, then the chunks of the remainder, which go first into the
 // places that the last round leaves.  64^3 FP32 (us a step): 4 planes 14.1, 3 planes
 // 17.9; 96^3: 12 planes 33.4, 6 planes 37.3; 128^3: 14 planes 74.9, 16 planes 79.8.
+// (FP32 windows: at most 32 planes and 1.2 more.)
+constexpr int kWindowPlanes = 32;
+constexpr double kWindowExtra = 1.2;
 double chunk_planes(long long xy, int nz, int places, int most, double extra, int* tz_out) {
   double best_cost = 1e300;
   for (int tz = 1; tz <= nz && tz <= most; ++tz) {
@@ -348,7 +353,7 @@ void tile_plan(lb_d3_handle* h, int sms) {
   h->tw = TX;
   h->th = TY;
   if (W::fixed) {
-    chunk_planes(tiles(TX, TY), nz, sms * d3_blocks<T>(), 32, 1.2, &h->tz);
+    chunk_planes(tiles(TX, TY), nz, sms * d3_blocks<T>(), kWindowPlanes, kWindowExtra, &h->tz);
     return;
   }
   double best = 1e300;
@@ -379,21 +384,46 @@ int chunk_planes_pull(int nx, int ny, int nz, int sms) {
   return tz;
 }
 
-// The step's windows by tensor copies where possible (FP32), else by 16-byte copies.
+// Whether an FP32 lattice steps faster by windows (k_d3_step) than by pulls (k_d3_pull), from
+// the planes that the last SM to finish works off.  Windows: chunk_planes.  Pulls: rounds of
+// 3 blocks per SM of tz planes and 2.5 more, the last one by half its fill and half whole; a
+// plane of a block of pulls costs more in the company of later rounds (sqrt(rounds)), and
+// windows lose what their 32 x 8 tiles hold outside the lattice.  The constant is from 160
+// lattices of 24 to 256 nodes a side, both forms timed on each: the form taken is the faster
+// or within 2% of it on 134, within 11% on all but one (120 x 124 x 33: 25.8 us, pulls 22.8).
+// Without the estimate, windows wherever the rows filled their tiles: 40^3 10.2 us a step
+// against 6.3 by pulls, 40 x 72 x 101 23.4 / 18.5, 104^3 57.0 / 50.2, 120 x 40 x 40 12.4 / 11.8, and
+// pulls at 196 x 35 x 48 21.2 / 19.1; windows are taken at 64^3 14.1 / 15.2, 96^3 33.9 / 41.2,
+// 160^3 133 / 152, 256^3 461 / 526.
+bool windows_win(int nx, int ny, int nz, int sms) {
+  const long long xy = (long long)((nx + TX - 1) / TX) * ((ny + TY - 1) / TY);
+  int tz = 1;
+  const double windows = chunk_planes(xy, nz, sms * d3_blocks<float>(), kWindowPlanes, kWindowExtra, &tz);
+  tz = chunk_planes_pull(nx, ny, nz, sms);
+  const long long places = 3LL * sms;
+  const long long blocks =
+      (long long)((nx + TX - 1) / TX) * ((ny + kPullTY - 1) / kPullTY) * ((nz + tz - 1) / tz);
+  const long long rounds = (blocks + places - 1) / places;
+  const double last = double(blocks - places * (rounds - 1)) / double(places);
+  const double pulls = (double(rounds) - 0.5 + 0.5 * last) * (tz + 2.5);
+  const double fill = double(nx) * ny / (double(xy) * TX * TY);
+  return windows < 0.37 * pulls * fill * std::sqrt(double(rounds));
+}
+
+// The step's windows by tensor copies where possible (FP32), else by 16-byte copies; FP32
+// rows that are no multiple of 16 bytes or shorter than a window (24 x 31 x 200: 11.5 us a step
+// against 13.3) take k_d3_pull.
 template <typename T>
-cudaError_t configure_step(lb_d3_handle* h) {
+cudaError_t configure_step(lb_d3_handle* h, int sms) {
   h->vec = (size_t(h->p.nx) * sizeof(T)) % 16 == 0 && reinterpret_cast<uintptr_t>(h->f[0]) % 16 == 0 &&
            reinterpret_cast<uintptr_t>(h->f[1]) % 16 == 0;
-  // FP32 lattices that k_d3_pull steps faster: rows that are no multiple of 16 bytes or
-  // shorter than a window (24 x 31 x 200: 11.5 us a step against 13.3), or so few of them
-  // that the last 32 x 8 tile is largely empty (160 x 12 x 80: 10.8 against 11.7; the
-  // windows gain 5 to 20% on full tiles).
-  const int rows8 = (h->p.ny + TY - 1) / TY * TY, rows4 = (h->p.ny + kPullTY - 1) / kPullTY * kPullTY;
-  h->windows = sizeof(T) == 8 || (h->vec && h->p.nx >= Win3<T>::cols && 10 * rows8 <= 11 * rows4);
+  h->can_window = sizeof(T) == 8 || (h->vec && h->p.nx >= Win3<T>::cols);
+  h->can_pull = sizeof(T) == 4;
+  h->auto_windows = h->can_window && (!h->can_pull || windows_win(h->p.nx, h->p.ny, h->nz, sms));
   h->have_maps = false;
   std::memset(h->maps, 0, sizeof(h->maps));
   using W = Win3<T>;
-  if (W::tensor && h->windows && h->p.ny >= W::rows) {
+  if (W::tensor && h->can_window && h->p.ny >= W::rows) {
     h->have_maps = true;
     for (int k = 0; k < 2; ++k)
       h->have_maps = h->have_maps &&
@@ -405,6 +435,25 @@ cudaError_t configure_step(lb_d3_handle* h) {
     e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k_d3_step<T, sizeof(T) != 8>),
                              cudaFuncAttributeMaxDynamicSharedMemorySize, int(Win3<T>::smem));
   return e;
+}
+
+void take_form(lb_d3_handle* h, bool windows) {
+  h->windows = windows;
+  if (!windows)
+    h->tz = chunk_planes_pull(h->p.nx, h->p.ny, h->nz, h->sms);
+  else if (h->p.precision == LB_FP64)
+    tile_plan<double>(h, h->sms);
+  else
+    tile_plan<float>(h, h->sms);
+}
+
+void drop_graphs(lb_d3_handle* h) {
+  for (int c = 0; c < 2; ++c) {
+    if (h->exec[c]) cudaGraphExecDestroy(h->exec[c]);
+    if (h->graph[c]) cudaGraphDestroy(h->graph[c]);
+    h->exec[c] = nullptr;
+    h->graph[c] = nullptr;
+  }
 }
 
 template <typename T, bool VEC>
@@ -573,14 +622,10 @@ int lb_d3_init(lb_d3_handle** out, const lb_params* p, int32_t nz, void* f_a, vo
     delete h;
     return cuda_fail(ce, what);
   };
-  e = q.precision == LB_FP64 ? configure_step<double>(h) : configure_step<float>(h);
+  e = q.precision == LB_FP64 ? configure_step<double>(h, sms) : configure_step<float>(h, sms);
   if (e != cudaSuccess) return give_up(e, "step configuration");
-  if (!h->windows)
-    h->tz = chunk_planes_pull(q.nx, q.ny, nz, sms);
-  else if (q.precision == LB_FP64)
-    tile_plan<double>(h, sms);
-  else
-    tile_plan<float>(h, sms);
+  h->sms = sms;
+  take_form(h, h->auto_windows);
   if (cudaMalloc(&h->part, (kReduceBlocks3 + 2) * kReduceSlots3 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     delete h;
@@ -666,6 +711,21 @@ int lb_d3_reduce(lb_d3_handle* h, double out[8]) {
   return LB_OK;
 }
 
+int lb_d3_form(const lb_d3_handle* h) { return !h ? LB_EINVAL : h->windows ? LB_D3_WINDOWS : LB_D3_PULLS; }
+
+int lb_d3_set_form(lb_d3_handle* h, int form) {
+  if (!h) return fail3(nullptr, LB_EINVAL, "null handle");
+  if (form != LB_D3_AUTO && form != LB_D3_PULLS && form != LB_D3_WINDOWS)
+    return fail3(h, LB_EINVAL, "form must be LB_D3_AUTO, LB_D3_PULLS or LB_D3_WINDOWS");
+  if ((form == LB_D3_PULLS && !h->can_pull) || (form == LB_D3_WINDOWS && !h->can_window))
+    return fail3(h, LB_ENOTSUP, "the lattice does not step in this form");
+  const bool windows = form == LB_D3_AUTO ? h->auto_windows : form == LB_D3_WINDOWS;
+  if (windows == h->windows) return LB_OK;
+  drop_graphs(h);  // captured with the other form
+  take_form(h, windows);
+  return LB_OK;
+}
+
 int lb_d3_status(lb_d3_handle* h) {
   if (!h) return fail3(nullptr, LB_EINVAL, "null handle");
   int v = 0;
@@ -705,10 +765,7 @@ const char* lb_d3_last_error(const lb_d3_handle* h) { return h ? h->err : thread
 
 void lb_d3_free(lb_d3_handle* h) {
   if (!h) return;
-  for (int c = 0; c < 2; ++c) {
-    if (h->exec[c]) cudaGraphExecDestroy(h->exec[c]);
-    if (h->graph[c]) cudaGraphDestroy(h->graph[c]);
-  }
+  drop_graphs(h);
   if (h->cstream) cudaStreamDestroy(h->cstream);
   if (h->part) cudaFree(h->part);
   delete h;

@@ -44,7 +44,7 @@ def _pair(shape, eos, Tr):
     """A two-phase lattice in FP32 and in FP64 with the same storage shift."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    from paper_1809_02390_gb300 import Lattice3
+    from paper_1809_02390_gb300 import Lattice3, capi
 
     nz, ny, nx = shape
     rng = np.random.default_rng(nx)
@@ -58,4 +58,8 @@ def _pair(shape, eos, Tr):
     wave = np.cos(2 * np.pi * (x / nx + y / ny)) + np.cos(2 * np.pi * (y / ny - z / nz) + 0.7)
     rho0 = 0.5 * (rho_g + rho_l) + 0.5 * (rho_l - rho_g) * np.tanh(1.2 * wave)
     rho0 *= 1 + 0.01 * rng.uniform(-1, 1, shape)
-    return (Lattice3(rho0, precision="fp32", rho_ref=ref, **kw), Lattice3(rho0, precision="fp64", rho_ref=ref, **kw))
+    lat = Lattice3(rho0, precision="fp32", rho_ref=ref, **kw)
+    if nx % 4 == 0:  # windows whatever the rule says of so small a lattice
+        capi.lb_d3_set_form(lat.h, capi.LB_D3_WINDOWS)
+    assert capi.lb_d3_form(lat.h) == (capi.LB_D3_WINDOWS if nx % 4 == 0 else capi.LB_D3_PULLS)
+    return lat, Lattice3(rho0, precision="fp64", rho_ref=ref, **kw)
