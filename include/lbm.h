@@ -134,8 +134,8 @@ size_t lb_state_bytes(const lb_params* p);
 /* Bytes of device scratch memory: one density plane (two-pass variant, reductions),
  * the reduction workspace, 256 bytes of tile tickets (fused tensor-copy step) and, for
  * lattices that fit the SMs' shared memory, the exchange words of the resident run
- * (lb_step; to 4 MB for squares, at most 18 MB for strips of three rows).  A buffer without the last part is accepted too: lb_step
- * then launches step by step. */
+ * (lb_step; to 4 MB for squares, at most 18 MB for strips of three rows).  A buffer without
+ * the last part is accepted too: lb_step then launches step by step. */
 size_t lb_scratch_bytes(const lb_params* p);
 
 /* Creates a handle bound to the caller's buffers and stream and initialises the
@@ -146,8 +146,9 @@ size_t lb_scratch_bytes(const lb_params* p);
  * that is not positive and finite (or, for vdW, not below 1/b) is reported.  f_a, f_b: device buffers of lb_state_bytes() each (ping-pong; f_a holds
  * the state after init).  scratch: device buffer of lb_scratch_bytes() bytes, or
  * NULL (the fused step then walks its tiles statically, and lb_reduce and the
- * two-pass variant are unavailable); it holds the tile tickets of the fused step,
- * so handles that step concurrently need scratch buffers of their own.  rho0: nx*ny doubles, row-major [y][x], on the host
+ * two-pass variant are unavailable); it holds the tile tickets of the fused step and
+ * the words of resident runs, so handles that step concurrently need scratch buffers of
+ * their own.  rho0: nx*ny doubles, row-major [y][x], on the host
  * (rho0_on_device = 0; copied through f_b, synchronously) or the device (1).
  * The handle keeps the pointers; the caller keeps ownership and must keep the
  * buffers alive until lb_free.  Fails with LB_EINVAL for bad parameters or
@@ -158,11 +159,13 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
             size_t scratch_bytes, const double* rho0, int rho0_on_device, void* stream);
 
 /* Advances nsteps >= 0 time steps (Eq. 13 + supplement Eq. 2) on the stream.
- * Asynchronous.  A small fused lattice (FP64 to 410^2, FP32 and FP16 to 340,000 nodes,
- * lb_step_form tells) takes calls of several steps (at least 4, FP32 and FP16 12) in one cooperative
- * launch that keeps it in the SMs' shared memory (same bits; waits between its blocks are
- * bounded at 10 s and reported by lb_status), unless lb_set_step_blocks or
- * lb_set_tile_dispatch asked for a tensor-copy form (lb_step_form tells which form serves a call).  Else runs of 64 steps replay a CUDA graph that the handle captures on
+ * Asynchronous.  A small fused lattice (FP64 to 410^2, FP32 and FP16 to 340,000 nodes) takes
+ * calls of several steps (at least 4, FP32 and FP16 12) in cooperative launches of about 5 ms
+ * that keep it in the SMs' shared memory (same bits; waits between blocks are bounded at 10 s
+ * and reported by lb_status), unless lb_set_resident, lb_set_step_blocks or lb_set_tile_dispatch
+ * say otherwise (lb_step_form tells which form serves a call) or more streams hold such lattices
+ * than runs of this one fit the GPU side by side.  A launch that the device refuses is replaced by
+ * ordinary ones.  Else runs of 64 steps replay a CUDA graph that the handle captures on
  * first use (again after lb_set_step_blocks or lb_set_tile_dispatch change the
  * launch); the graph runs on a stream the handle owns, ordered after the caller's
  * stream's earlier work and before its later work, and gives the same bits as 64

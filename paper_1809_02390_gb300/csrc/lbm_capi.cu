@@ -196,9 +196,12 @@ constexpr size_t kQueueBytes = 256;  // tile tickets of the dynamic tensor-copy 
 // steps are then launched one by one).
 size_t base_scratch_bytes(const lb_params* p) { return rho_plane_bytes(p) + reduce_bytes() + kQueueBytes; }
 
-// Fewest steps of a call that run resident: the launch costs some 8 us more than an
-// ordinary one (load, store, cooperative start), a step less (FP32 256^2 2.15 against 2.74 us,
-// 400^2 3.0 / 4.2, FP16 256^2 2.5 / 3.35: from 12 or 13, 8 and 8 steps; FP64 64^2 7.6 / 21.5).
+// Fewest steps of a call that run resident: the launch costs 7 to 10 us more than an
+// ordinary one (load, store, cooperative start), a step less.  Calls of single launches
+// against resident ones, us a step (FP32 256^2 2.51 against 2.91 in calls of 12 steps, 2.70 of 16,
+// 2.31 of 40, 2.18 of 130; 301^2 3.00 / 3.08, 2.95, 2.62, 2.47; 512^2 4.77 / 4.79, 4.52, 4.15, 3.98;
+// FP16 301^2 3.87 / 3.59, 3.34, 3.08, 2.92; FP64 64^2 16.3 / 9.25 in calls of 4, 8.38 of 11).  The line
+// of 12 is that of the larger lattices; FP32 128^2 gains from some 40 steps on, 256^2 from 24.
 int64_t res_min_steps(const lb_handle* h) { return h->p.precision == LB_FP64 ? 4 : 12; }
 // The same for runs that record states.
 int64_t res_min_record(const lb_handle* h) { return h->p.precision == LB_FP64 ? 2 : 12; }

@@ -151,7 +151,7 @@ cudaError_t res_configure(lb_handle* h, void* mail) {
   ResPlan p;
   // FP32 and FP16 up to kResNodes: above, a tile's pitch no longer avoids bank conflicts
   // and a step is no faster than a launch of k_step_fused (us: FP32 576^2 4.9 against 5.3,
-  // 600^2 6.8 / 5.7; FP16 480^2 4.7 / 4.9, 576^2 6.0 / 6.3, 640 x 600 7.0 / 6.7, 800^2 10.8 / 9.8).
+  // 600^2 6.8 / 5.6; FP16 400^2 3.8 / 3.9, 512^2 5.2 / 4.7, 576^2 6.0 / 6.2, 640 x 600 7.0 / 6.6).
   if (h->p.precision != LB_FP64 && (long long)h->p.nx * h->p.ny > kResNodes) return cudaSuccess;
   if (!mail || h->variant != LB_FUSED || !res_plan(h->p.nx, h->p.ny, h->p.precision, &p)) return cudaSuccess;
   const void* k = res_kernel(h->p.precision);

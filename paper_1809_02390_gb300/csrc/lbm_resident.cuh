@@ -2,11 +2,11 @@
 // is cut into at most one tile per SM, a tile's populations stay in its SM's shared
 // memory for all steps, and only the edges travel between SMs.
 //
-// What bounds short steps: with one launch per step (graph replay) a 256^2 FP32 step
-// takes 4.1 us, of which the collision is about 0.7 us; the rest is launch latency,
-// the round trip of every population through L2 and the drain between launches.
-// Here a step costs the collision, three block barriers and one exchange: 2.15 us at
-// 256^2, 3.9 us at 512^2 (7.6 us by graph), FP64 64^2 7.7 us (33.8 us).  What is left
+// What bounds short steps: with one launch per step (graph replay, launches that overlap)
+// a 256^2 FP32 step takes 2.4 us, of which the collision is about 0.7 us; the rest is launch
+// latency, the round trip of every population through L2 and the drain between launches.
+// Here a step costs the collision, three block barriers and one exchange: 2.12 us at
+// 256^2, 3.9 us at 512^2 (4.5 us by graph), FP64 64^2 7.7 us (15.9 us).  What is left
 // at 256^2 (cycles): collision of the edge nodes 1500, sending them 600, the trip
 // through L2 1200 to 1500, densities 400, barriers 200.  From about 400^2 on the
 // collisions' issue bounds it.  Measured and not kept: 768 threads at 80 registers
@@ -31,7 +31,8 @@
 // What the scratch buffer held before a run is never taken for a word of it: every tile
 // clears its own words first, and no tile reads any before all tiles have (a grid barrier,
 // arrived at right after clearing and waited for once the tile is loaded; waiting in the
-// second step instead kept its state alive in the loop, 2.17 us a step at 256^2).  So handles that share a scratch buffer may run in turn, whatever they left in it.
+// second step instead kept its state alive in the loop, 2.17 us a step at 256^2).  So handles
+// that share a scratch buffer may run in turn, whatever they left in it.
 #pragma once
 
 #include <cooperative_groups.h>
