@@ -163,8 +163,8 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
  * calls of several steps (at least 4, FP32 and FP16 12) in cooperative launches of about 5 ms
  * that keep it in the SMs' shared memory (same bits; waits between blocks are bounded at 10 s
  * and reported by lb_status), unless lb_set_resident, lb_set_step_blocks or lb_set_tile_dispatch
- * say otherwise (lb_step_form tells which form serves a call) or more streams hold such lattices
- * than runs of this one fit the GPU side by side.  A launch that the device refuses is replaced by
+ * say otherwise (lb_step_form tells which form serves a call) or lattices on more streams make
+ * such calls than runs of this one fit the GPU side by side.  A launch that the device refuses is replaced by
  * ordinary ones.  Else runs of 64 steps replay a CUDA graph that the handle captures on
  * first use (again after lb_set_step_blocks or lb_set_tile_dispatch change the
  * launch); the graph runs on a stream the handle owns, ordered after the caller's
@@ -401,8 +401,8 @@ int lb_step_form(const lb_handle* h, int64_t nsteps);
  * lattice fits and a call has steps enough.  Resident runs hold their SMs to the end, so
  * lattices that step on streams of their own take turns once the GPU is full, where single
  * launches share it; the rule therefore leaves resident runs while more streams of the device
- * hold live handles of such lattices than runs of this one fit the GPU side by side (FP32
- * 64^2 five, 256^2 two, 512^2 one).  Same bits either way.  LB_ENOTSUP for 1 where the lattice
+ * hold live handles that have made calls long enough for them than runs of this one fit the
+ * GPU side by side (FP32 64^2 five, 256^2 two, 512^2 one).  Same bits either way.  LB_ENOTSUP for 1 where the lattice
  * or its scratch buffer does not allow it, LB_EINVAL for other values. */
 int lb_set_resident(lb_handle* h, int mode);
 

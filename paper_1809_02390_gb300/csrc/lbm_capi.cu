@@ -215,7 +215,7 @@ int launch_form(const lb_handle* h) {
 }
 
 // Whether a call of nsteps steps runs resident (outside a capture): from `least` steps on,
-// while the streams that hold lattices which could are no more than the runs of this one that
+// while the streams whose lattices make such calls are no more than the runs of this one that
 // fit the GPU side by side, or as lb_set_resident says.  A run beyond those waits for a whole
 // launch of another, while single launches share the GPU (us a step of k lattices on k streams,
 // resident / graphs of k_step_fused: FP32 64^2, 5 fit: k = 4 2.1 / 2.2, 6 4.0 / 2.3; 200 x 180, 3
@@ -225,6 +225,10 @@ int launch_form(const lb_handle* h) {
 bool resident_call(const lb_handle* h, int64_t nsteps, int64_t least) {
   if (!h->use_res || h->forced_blocks || h->forced_dispatch || h->res_mode == 0 || nsteps < least) return false;
   return h->res_mode == 1 || res_streams(h) <= h->res_fit;
+}
+bool take_resident(lb_handle* h, int64_t nsteps, int64_t least) {
+  if (h->use_res && nsteps >= least) res_enter(h);
+  return resident_call(h, nsteps, least);
 }
 
 template <typename V, typename real, typename store_t>
@@ -657,7 +661,6 @@ int lb_init(lb_handle** out, const lb_params* p, void* f_a, void* f_b, void* scr
   h->c2 = make_vcoef<f2>(h->p, d);
   h->cd = make_vcoef<double>(h->p, d);
   h->wait_slot = -1;
-  h->res_dev = -1;
   h->graph_k = -1;
   rc = configure(h);
   if (rc != LB_OK) {
@@ -813,7 +816,7 @@ int lb_step(lb_handle* h, int64_t nsteps) {
     capture = cudaStreamCaptureStatusActive;  // unknown: take the plain launches
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_steps(h))) {
+  if (capture == cudaStreamCaptureStatusNone && take_resident(h, nsteps, res_min_steps(h))) {
     int64_t done = 0;
     LB_CUDA(h, res_run(h, nsteps, nullptr, 1, &done));
     nsteps -= done;  // none left, unless the device refused a launch
@@ -861,7 +864,7 @@ int lb_step_record(lb_handle* h, int64_t nsteps, int64_t every, void* states) {
     capture = cudaStreamCaptureStatusActive;
   }
   h->overlap = capture == cudaStreamCaptureStatusNone;
-  if (capture == cudaStreamCaptureStatusNone && resident_call(h, nsteps, res_min_record(h)) &&
+  if (capture == cudaStreamCaptureStatusNone && take_resident(h, nsteps, res_min_record(h)) &&
       record_by_elements(h->p, reinterpret_cast<uintptr_t>(at))) {
     int64_t done = 0;
     LB_CUDA(h, res_run(h, nsteps, states, every, &done));

@@ -59,7 +59,8 @@ struct lb_handle {
   int res_mode;           // lb_set_resident: -1 by rule, 0 never, 1 always
   int res_fit;            // resident runs of this lattice that fit the GPU side by side
   int64_t res_refuse;     // lb_resident_selftest: launches until one is taken for refused (-1: none)
-  int res_dev;            // device of the handle's entry among the live resident handles (-1: none)
+  int res_dev;            // device
+  bool res_live;          // the handle counts among those that step resident (res_enter)
   void* res_mail;         // exchange words (end of the scratch buffer)
   unsigned* step_word;    // device word with the step count a replayed FP16 graph seeds from
   bool overlap;           // the steps' launches may overlap their predecessor's end (lbm_launch.cuh)
@@ -90,9 +91,11 @@ size_t res_mail_bytes(int nx, int ny);
 // Decides whether the handle can run resident with the exchange buffer `mail` (device
 // memory of res_mail_bytes, 16-byte aligned, or null; its contents do not matter).
 cudaError_t res_configure(lb_handle* h, void* mail);
-// Takes the handle out of the live ones (lb_free).
+// Counts the handle among those that step resident (its first call that is long enough),
+// and takes it out again (lb_free).
+void res_enter(lb_handle* h);
 void res_leave(lb_handle* h);
-// Streams of the handle's device that live handles which can run resident are bound to.
+// Streams of the handle's device that counted handles are bound to, its own included.
 int res_streams(const lb_handle* h);
 // Advances the handle's lattice by nsteps >= 2 steps and its counters with it; rec (or
 // null): device memory that receives the states after every `every` steps.

@@ -101,8 +101,9 @@ size_t res_mail_bytes(int nx, int ny) {
 }
 
 namespace {
-// Live handles that can run resident, by device and stream (an entry goes with its last
-// handle), and the number of streams per device, which every step call reads.
+// Live handles that have made a call long enough to run resident, by device and stream (an
+// entry goes with its last handle), and the number of streams per device, which every step
+// call reads.
 struct Live {
   int dev;
   cudaStream_t stream;
@@ -113,21 +114,27 @@ std::mutex g_live_mu;
 std::vector<Live> g_live;
 std::atomic<int> g_live_streams[kDevices];
 
-void res_enter(lb_handle* h, int dev) {
-  std::lock_guard<std::mutex> lock(g_live_mu);
-  h->res_dev = dev;
+Live* find_live(const lb_handle* h) {
   for (Live& l : g_live)
-    if (l.dev == dev && l.stream == h->stream) {
-      ++l.handles;
-      return;
-    }
-  g_live.push_back(Live{dev, h->stream, 1});
-  ++g_live_streams[dev % kDevices];
+    if (l.dev == h->res_dev && l.stream == h->stream) return &l;
+  return nullptr;
 }
 }  // namespace
 
+void res_enter(lb_handle* h) {
+  if (h->res_live) return;
+  std::lock_guard<std::mutex> lock(g_live_mu);
+  h->res_live = true;
+  if (Live* l = find_live(h)) {
+    ++l->handles;
+    return;
+  }
+  g_live.push_back(Live{h->res_dev, h->stream, 1});
+  ++g_live_streams[h->res_dev % kDevices];
+}
+
 void res_leave(lb_handle* h) {
-  if (!h || h->res_dev < 0) return;
+  if (!h || !h->res_live) return;
   std::lock_guard<std::mutex> lock(g_live_mu);
   for (size_t k = 0; k < g_live.size(); ++k)
     if (g_live[k].dev == h->res_dev && g_live[k].stream == h->stream) {
@@ -137,11 +144,14 @@ void res_leave(lb_handle* h) {
       }
       break;
     }
-  h->res_dev = -1;
+  h->res_live = false;
 }
 
 int res_streams(const lb_handle* h) {
-  return h->res_dev < 0 ? 0 : g_live_streams[h->res_dev % kDevices].load(std::memory_order_relaxed);
+  const std::atomic<int>& streams = g_live_streams[h->res_dev % kDevices];
+  if (h->res_live) return streams.load(std::memory_order_relaxed);
+  std::lock_guard<std::mutex> lock(g_live_mu);
+  return streams.load(std::memory_order_relaxed) + (find_live(h) ? 0 : 1);
 }
 
 cudaError_t res_configure(lb_handle* h, void* mail) {
@@ -167,8 +177,8 @@ cudaError_t res_configure(lb_handle* h, void* mail) {
   h->res = p;
   h->res_mail = mail;
   h->res_fit = per_sm * sms / (p.gx * p.gy);
+  h->res_dev = dev;
   h->use_res = true;
-  res_enter(h, dev);
   return cudaSuccess;
 }
 

@@ -1,6 +1,6 @@
-"""Resident runs and several streams: while more streams hold lattices that fit than runs of
-one fit the GPU side by side, calls take single launches again; lb_set_resident decides
-otherwise.  The bits are the same."""
+"""Resident runs and several streams: while lattices on more streams make long calls than runs
+of one fit the GPU side by side, calls take single launches again; lb_set_resident decides
+otherwise.  Lattices that make none do not count.  The bits are the same."""
 import pytest
 
 from paper_1809_02390_gb300 import inputs
@@ -32,8 +32,15 @@ def test_many_streams_leave_resident_runs(precision):
     lats = _lats([one], precision=precision)
     assert capi.lb_step_form(lats[0].h, 40) == R
     lats += _lats([one] * 12, precision=precision)  # many lattices, one stream
+    for lat in lats:
+        lat.step(40)
     assert all(capi.lb_step_form(lat.h, 40) == R for lat in lats)
     others = [_lats([torch.cuda.Stream()], precision=precision)[0] for _ in range(12)]
+    for lat in others:
+        lat.step(3)  # too short for a resident run
+    assert all(capi.lb_step_form(lat.h, 40) == R for lat in lats)
+    for lat in others:
+        lat.step(37)
     assert all(capi.lb_step_form(lat.h, 40) == capi.LB_STEP_PLAIN for lat in lats + others)
     capi.lb_set_resident(others[3].h, 1)
     assert capi.lb_step_form(others[3].h, 40) == R
@@ -42,7 +49,7 @@ def test_many_streams_leave_resident_runs(precision):
     for _ in range(3):
         for lat in others:
             lat.step(40)
-    for _ in range(120):
+    for _ in range(160):
         ref.step(1)
     torch.cuda.synchronize()
     for lat in others:
