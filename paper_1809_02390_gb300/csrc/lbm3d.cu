@@ -388,9 +388,10 @@ int chunk_planes_pull(int nx, int ny, int nz, int sms) {
 // the planes that the last SM to finish works off.  Windows: chunk_planes.  Pulls: rounds of
 // 3 blocks per SM of tz planes and 2.5 more, the last one by half its fill and half whole; a
 // plane of a block of pulls costs more in the company of later rounds (sqrt(rounds)), and
-// windows lose what their 32 x 8 tiles hold outside the lattice.  The constant is from 160
+// windows lose what their 32 x 8 tiles hold outside the lattice.  The constant is from 159
 // lattices of 24 to 256 nodes a side, both forms timed on each: the form taken is the faster
-// or within 2% of it on 134, within 11% on all but one (120 x 124 x 33: 25.8 us, pulls 22.8).
+// or within 2% of it on 140, within 9% on all but two (120 x 124 x 33: 25.8 us, pulls 22.8;
+// 240 x 160 x 48: 76.0, windows 67.8).
 // Without the estimate, windows wherever the rows filled their tiles: 40^3 10.2 us a step
 // against 6.3 by pulls, 40 x 72 x 101 23.4 / 18.5, 104^3 57.0 / 50.2, 120 x 40 x 40 12.4 / 11.8, and
 // pulls at 196 x 35 x 48 21.2 / 19.1; windows are taken at 64^3 14.1 / 15.2, 96^3 33.9 / 41.2,
